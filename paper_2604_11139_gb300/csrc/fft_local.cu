@@ -26,6 +26,7 @@
 #include <utility>
 
 #include "pw_internal.cuh"
+#include "fft_fixed.cuh"
 
 namespace pw {
 
@@ -2963,6 +2964,10 @@ cudaError_t launch_local_apply(const FftPlan& plan, const cplx<T>* tw, const Sph
                                int nband, cplx<T>* out, int64_t ldout, cplx<T>* hb, int band_batch,
                                cudaStream_t st, ::pw_ctx* prof) {
   if (nband <= 0) return cudaSuccess;
+  if constexpr (std::is_same<T, double>::value) {
+    if (fx::covers(plan))
+      return fx::local_apply(plan, tw, sp, vperm, kin, psi, ldpsi, nband, out, ldout, hb, band_batch, st, prof);
+  }
   const int cz = pick_cz(plan.n[2]);
   const int lyz = 32;
   const size_t sm1 = plane_smem<T>(plan, sp, cz);
@@ -3276,6 +3281,12 @@ cudaError_t launch_density(const FftPlan& plan, const cplx<T>* tw, const SphereD
                            const cplx<T>* a, const cplx<T>* b, int64_t ld, int nband, const T* w_dev,
                            double* out_perm, cplx<T>* hb, int band_batch, cudaStream_t st) {
   if (nband <= 0) return cudaSuccess;
+  if constexpr (std::is_same<T, double>::value) {
+    if (fx::covers(plan)) {
+      const cudaError_t fe = fx::density(plan, tw, sp, a, b, ld, nband, w_dev, out_perm, hb, band_batch, st);
+      if (fe != cudaErrorNotSupported) return fe;
+    }
+  }
   const int cz = pick_cz(plan.n[2]);
   const int lyz = 8;  // 8 accumulators per thread cover n1*lyz <= 2048 points
   if (plan.n[0] * lyz > 8 * kThreads) return cudaErrorInvalidValue;

@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "la.cuh"
+#include "fft_fixed.cuh"
 #include "pw_internal.cuh"
 #include "setup.cuh"
 #include "tc.cuh"
@@ -1408,8 +1409,9 @@ int create_impl(const pw_problem_desc* d, void* stream, pw_ctx** out) {
   PW_TRY(upload(ctx, &ctx->kin64, ctx->kin_h.data(), ctx->kin_h.size()));
   std::vector<float> kin32(ctx->kin_h.begin(), ctx->kin_h.end());
   PW_TRY(upload(ctx, &ctx->kin32, kin32.data(), kin32.size()));
-  // twiddles e^{-2 pi i j m / L}
+  // twiddles e^{-2 pi i j m / L}; the fixed-point table of the complex128 passes has the same layout
   std::vector<double2> tw;
+  std::vector<fx::Tw> twf;
   for (int dd = 0; dd < 3; ++dd) {
     FftDim& f = ctx->plan.d[dd];
     f.tw_base = (int)tw.size();
@@ -1421,12 +1423,16 @@ int create_impl(const pw_problem_desc* d, void* stream, pw_ctx** out) {
           const long jm = ((long)j * m) % L;
           const double ang = -2.0 * kPi * (double)jm / (double)L;
           tw.push_back(make_double2(cos(ang), sin(ang)));
+          twf.push_back(fx::twiddle(jm, L));
         }
     }
     f.tw_count = (int)tw.size() - f.tw_base;
   }
   std::vector<float2> tw32(tw.size());
   for (size_t i = 0; i < tw.size(); ++i) tw32[i] = make_float2((float)tw[i].x, (float)tw[i].y);
+  ctx->plan.tw_total = (int)tw.size();
+  tw.resize(2 * twf.size());  // the FP64 table, then the fixed-point one
+  if (!twf.empty()) memcpy(tw.data() + twf.size(), twf.data(), sizeof(fx::Tw) * twf.size());
   PW_TRY(upload(ctx, &ctx->tw64, tw.data(), tw.size()));
   PW_TRY(upload(ctx, &ctx->tw32, tw32.data(), tw32.size()));
   for (int dd = 0; dd < 3; ++dd) {

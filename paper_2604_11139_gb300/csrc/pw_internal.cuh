@@ -75,6 +75,7 @@ struct FftDim {
 struct FftPlan {
   int n[3];
   FftDim d[3];
+  int tw_total;  // entries of the twiddle table over all dimensions
 };
 
 // Radix plan of one FFT length, shared by host and device code.  Stages use the
