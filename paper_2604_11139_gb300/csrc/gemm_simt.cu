@@ -118,6 +118,48 @@ __global__ void __launch_bounds__(256) k_cgemm(int M, int N, int K, const cplx<T
   }
 }
 
+// 16 x 16 tiles, one output per thread: products whose 64 x 64 tiles leave SMs without work (the
+// subspace matrices of a few hundred bands).  FP64 issues at 2 lanes per clock and SM, so a large
+// tile takes its SM 256 K clocks whatever feeds it: 512^3 2.06 ms on 64 tiles of 64 and 0.91 ms on
+// 1024 of 16; complex64 at 64 x 37 x 64 13 and 3.5 us.  Same order of the sum over K as the large tiles without split.
+template <typename T, int TA, int TB>
+__global__ void __launch_bounds__(256) k_cgemm16(int M, int N, int K, const cplx<T>* __restrict__ A, int64_t lda,
+                                                 const cplx<T>* __restrict__ B, int64_t ldb, Epi<T> epi, int tri) {
+  using C = cplx<T>;
+  __shared__ C As[16][17], Bs[16][17];
+  const int x = threadIdx.x & 15, y = threadIdx.x >> 4;
+  const int m0 = blockIdx.x * 16, n0 = blockIdx.y * 16;
+  if (tri == GEMM_LOWER_OUT && m0 / BM < n0 / BN) return;  // tile above the diagonal
+  const int ke = tri == GEMM_B_UPPER ? min(K, n0 + 16) : K;  // op(B)[k][n] = 0 for k > n
+  C acc = czero<C>();
+  for (int k0 = 0; k0 < ke; k0 += 16) {
+    {
+      const int gm = m0 + (TA ? y : x), gk = k0 + (TA ? x : y);
+      C v = czero<C>();
+      if (gm < M && gk < ke) v = TA ? cconj(A[gk + (int64_t)gm * lda]) : A[gm + (int64_t)gk * lda];
+      As[TA ? x : y][TA ? y : x] = v;
+    }
+    {
+      const int gn = n0 + (TB ? x : y), gk = k0 + (TB ? y : x);
+      C v = czero<C>();
+      if (gn < N && gk < ke) v = TB ? cconj(B[gn + (int64_t)gk * ldb]) : B[gk + (int64_t)gn * ldb];
+      Bs[TB ? y : x][TB ? x : y] = v;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      const C a = As[k][x], b = Bs[k][y];
+      acc.x = fma(a.x, b.x, acc.x);
+      acc.x = fma(-a.y, b.y, acc.x);
+      acc.y = fma(a.x, b.y, acc.y);
+      acc.y = fma(a.y, b.x, acc.y);
+    }
+    __syncthreads();
+  }
+  const int m = m0 + x, n = n0 + y;
+  if (m < M && n < N) epi_apply<T>(epi, m, n, acc);
+}
+
 template <typename T>
 __global__ void k_splitk_reduce(int M, int N, int nsplit, const cplx<T>* __restrict__ ws, Epi<T> epi, int tri) {
   using C = cplx<T>;
@@ -176,38 +218,48 @@ __global__ void __launch_bounds__(256) k_cgemv_t(int M, int K, const cplx<T>* __
   }
 }
 
-// out[i][j] = sum_k A[i][k] B[k][j]: one thread per row i, B's few columns broadcast; the K
-// loop is unrolled so that several rows of A are in flight per thread
+// out[i][j] = sum_k A[i][k] B[k][j]: 64 rows per CTA, K in 4 interleaved parts (18.6 us at 14771 x
+// 136 FP64; CTAs of 256 rows leave most SMs without work there, 36 us); the K loop is unrolled so that several
+// rows of A are in flight per thread
 template <typename T, int NB>
 __global__ void __launch_bounds__(256) k_cgemv_n(int M, int K, const cplx<T>* __restrict__ A, int64_t lda,
                                                  const cplx<T>* __restrict__ B, int64_t ldb, Epi<T> epi) {
   using C = cplx<T>;
-  const int i = blockIdx.x * 256 + threadIdx.x;
-  if (i >= M) return;
+  __shared__ C red[4][NB][64];
+  const int r = threadIdx.x & 63, q = threadIdx.x >> 6;
+  const int i = blockIdx.x * 64 + r;
   C acc[NB];
 #pragma unroll
   for (int j = 0; j < NB; ++j) acc[j] = czero<C>();
+  if (i < M) {
 #pragma unroll 8
-  for (int k = 0; k < K; ++k) {
-    const C x = A[i + (int64_t)k * lda];
+    for (int k = q; k < K; k += 4) {
+      const C x = A[i + (int64_t)k * lda];
 #pragma unroll
-    for (int j = 0; j < NB; ++j) {
-      const C b = B[k + (int64_t)j * ldb];
-      acc[j].x = fma(x.x, b.x, acc[j].x);
-      acc[j].x = fma(-x.y, b.y, acc[j].x);
-      acc[j].y = fma(x.x, b.y, acc[j].y);
-      acc[j].y = fma(x.y, b.x, acc[j].y);
+      for (int j = 0; j < NB; ++j) {
+        const C b = B[k + (int64_t)j * ldb];
+        acc[j].x = fma(x.x, b.x, acc[j].x);
+        acc[j].x = fma(-x.y, b.y, acc[j].x);
+        acc[j].y = fma(x.x, b.y, acc[j].y);
+        acc[j].y = fma(x.y, b.x, acc[j].y);
+      }
     }
   }
 #pragma unroll
-  for (int j = 0; j < NB; ++j) epi_apply<T>(epi, i, j, acc[j]);
+  for (int j = 0; j < NB; ++j) red[q][j][r] = acc[j];
+  __syncthreads();
+  if (q == 0 && i < M) {
+#pragma unroll
+    for (int j = 0; j < NB; ++j)
+      epi_apply<T>(epi, i, j, cadd(cadd(red[0][j][r], red[1][j][r]), cadd(red[2][j][r], red[3][j][r])));
+  }
 }
 
 template <typename T, int NB>
 static void launch_gemv(int ta, int M, int K, const cplx<T>* A, int64_t lda, const cplx<T>* B, int64_t ldb,
                         const Epi<T>& epi, cudaStream_t st) {
   if (ta == 1) k_cgemv_t<T, NB><<<M, 256, 0, st>>>(M, K, A, lda, B, ldb, epi);
-  else k_cgemv_n<T, NB><<<(M + 255) / 256, 256, 0, st>>>(M, K, A, lda, B, ldb, epi);
+  else k_cgemv_n<T, NB><<<(M + 63) / 64, 256, 0, st>>>(M, K, A, lda, B, ldb, epi);
   count_launch();
 }
 
@@ -235,6 +287,18 @@ cudaError_t launch_cgemm(int ta, int tb, int M, int N, int K, const cplx<T>* A, 
   nsplit = (K + kchunk - 1) / kchunk;
   if (nsplit < 1) nsplit = 1;
   const int tm = (M + BM - 1) / BM, tn = (N + BN - 1) / BN;
+  // without split: 16 x 16 tiles while the 64 x 64 ones do not give every SM one.  FP64: always the
+  // better there; FP32 reuses an operand from registers 4 times in the large tile, which pays from
+  // about 16 tiles on
+  if (nsplit == 1 && K > 0 && tm * tn < (sizeof(T) == 8 ? 152 : 16)) {
+    const dim3 g((M + 15) / 16, (N + 15) / 16);
+    if (ta == 0 && tb == 0) k_cgemm16<T, 0, 0><<<g, 256, 0, st>>>(M, N, K, A, lda, B, ldb, epi, tri);
+    else if (ta == 1 && tb == 0) k_cgemm16<T, 1, 0><<<g, 256, 0, st>>>(M, N, K, A, lda, B, ldb, epi, tri);
+    else if (ta == 0 && tb == 1) k_cgemm16<T, 0, 1><<<g, 256, 0, st>>>(M, N, K, A, lda, B, ldb, epi, tri);
+    else k_cgemm16<T, 1, 1><<<g, 256, 0, st>>>(M, N, K, A, lda, B, ldb, epi, tri);
+    count_launch();
+    return cudaGetLastError();
+  }
   dim3 grid(tm, tn, nsplit);
   if (tri == GEMM_LOWER_OUT) grid = dim3(tm * (tm + 1) / 2, 1, nsplit);
   if (ta == 0 && tb == 0) k_cgemm<T, 0, 0><<<grid, 256, 0, st>>>(M, N, K, A, lda, B, ldb, epi, kchunk, ws, tri);

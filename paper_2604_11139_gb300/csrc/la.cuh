@@ -27,9 +27,11 @@ cudaError_t la_coldot(const double2* A, int64_t lda, const double2* B, int64_t l
 cudaError_t la_resid(const double2* HY, int64_t ldh, const double2* SY, int64_t lds, int npw, int m,
                      const double* eig, double* r, cudaStream_t st);
 cudaError_t la_rq_minmax(const double2* num, const double2* den, int m, double* rq, double* mm, cudaStream_t st);
-// steps-step Lanczos from v0; ab: 2*steps doubles; bound: 2 doubles {theta+|beta|, theta}
+// steps-step Lanczos from v0; ab: 2*steps doubles; bound: 2 doubles {theta+|beta|, theta};
+// part: 2 * la_lz_blocks doubles
+constexpr int la_lz_blocks = 152;
 cudaError_t la_lanczos(const double2* v0, int n, int steps, double2* v, double2* vprev, double2* w, double* ab,
-                       double* bound, ApplyFn apply, void* ctx, cudaStream_t st);
+                       double* bound, double* part, ApplyFn apply, void* ctx, cudaStream_t st);
 cudaError_t la_to_c64(const double2* a, int64_t lda, float2* b, int64_t ldb, int n, int m, cudaStream_t st);
 cudaError_t la_to_c128(const float2* a, int64_t lda, double2* b, int64_t ldb, int n, int m, cudaStream_t st);
 // LOBPCG: W = K (HX - lam SX) with the Teter-Payne-Allan preconditioner, rn = residual norms

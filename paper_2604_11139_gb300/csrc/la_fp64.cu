@@ -49,77 +49,90 @@ cudaError_t la_herm_from_lower(double2* A, int64_t lda, int n, cudaStream_t st) 
 // ---- blocked Cholesky A = L L^dagger (lower, in place; strict upper part zeroed) ---
 constexpr int NB = 32;
 
-__global__ void k_chol_diag(double2* A, int64_t lda, int k0, int kb, int* flag) {
-  __shared__ double2 S[NB][NB + 1];
-  const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 32
-  if (tx < kb && ty < kb) S[ty][tx] = A[(k0 + ty) + (int64_t)(k0 + tx) * lda];  // S[row][col]
+// One panel: every CTA factors the 32 x 32 diagonal block for itself, in shared memory, and solves its kPR rows below, L21[i,:] = A21[i,:] L11^{-dagger}, one row per warp.
+// FP64 issues at 2 lanes per clock and SM, so the work is spread over as many SMs as it has rows /
+// 8, with the columns of a row over the lanes.  n = 512: 73 us a panel, the diagonal
+// block's chain of square roots, divisions and updates; 75 + 131 us in two launches (1 CTA, and a
+// thread per row on 4 CTAs) before.
+// The other CTAs may still read the block, so CTA 0 leaves its factor where they do not look: the
+// strict lower part mirrored into the block's strict upper part, the diagonal in the imaginary
+// parts of A's (k_chol_finish puts them in place).
+constexpr int kPR = 8;
+__global__ void __launch_bounds__(256) k_chol_panel(double2* A, int64_t lda, int n, int k0, int kb, int* flag) {
+  __shared__ double2 S[NB][NB + 1];  // S[col][row]
+  __shared__ double inv[NB];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  for (int e = t; e < NB * NB; e += 256) {
+    const int r = e % NB, c = e / NB;
+    double2 v = make_double2(0.0, 0.0);
+    if (r < kb && c < r) v = A[(k0 + r) + (int64_t)(k0 + c) * lda];
+    if (r < kb && c == r) v.x = A[(k0 + r) + (int64_t)(k0 + r) * lda].x;
+    S[c][r] = v;
+  }
   __syncthreads();
   for (int j = 0; j < kb; ++j) {
-    if (tx == 0 && ty == 0) {
+    if (w == 0) {
       double d = S[j][j].x;
-      if (!(d > 0.0) || !isfinite(d)) { atomicExch(flag, 1); d = 1.0; }
-      S[j][j] = make_double2(sqrt(d), 0.0);
+      const bool bad = !(d > 0.0) || !isfinite(d);
+      if (bad) d = 1.0;
+      const double s = sqrt(d), i = 1.0 / s;
+      if (lane > j && lane < kb) S[j][lane] = cscale(S[j][lane], i);
+      __syncwarp();
+      if (lane == 0) {
+        if (bad && blockIdx.x == 0) atomicExch(flag, 1);
+        S[j][j] = make_double2(s, 0.0);
+        inv[j] = i;
+      }
     }
     __syncthreads();
-    const double dj = S[j][j].x;
-    if (tx == 0 && ty > j && ty < kb) S[ty][j] = cscale(S[ty][j], 1.0 / dj);
-    __syncthreads();
-    // trailing: S[i][k] -= S[i][j] conj(S[k][j]) for j < k <= i
-    if (ty > j && ty < kb && tx > j && tx <= ty) S[ty][tx] = csub(S[ty][tx], cmul(S[ty][j], cconj(S[tx][j])));
+    // S[k][i] -= S[j][i] conj(S[j][k]) for j < k <= i: lane = row, the warps take the columns
+    for (int k = j + 1 + w; k < kb; k += 8)
+      if (lane >= k && lane < kb) S[k][lane] = csub(S[k][lane], cmul(S[j][lane], cconj(S[j][k])));
     __syncthreads();
   }
-  if (tx < kb && ty < kb) {
-    const double2 v = (tx <= ty) ? S[ty][tx] : make_double2(0.0, 0.0);
-    A[(k0 + ty) + (int64_t)(k0 + tx) * lda] = v;
-  }
-}
-
-// rows i >= k0+kb: L21[i,:] = A21[i,:] L11^{-dagger}
-__global__ void k_chol_panel(double2* A, int64_t lda, int n, int k0, int kb) {
-  __shared__ double2 Ls[NB][NB + 1];
-  const int t = threadIdx.x;
-  for (int e = t; e < kb * kb; e += blockDim.x) {
-    const int r = e % kb, c = e / kb;
-    Ls[r][c] = A[(k0 + r) + (int64_t)(k0 + c) * lda];
-  }
-  __syncthreads();
-  const int i = k0 + kb + blockIdx.x * blockDim.x + t;
+  if (blockIdx.x == 0)
+    for (int e = t; e < NB * NB; e += 256) {
+      const int r = e % NB, c = e / NB;
+      if (r >= kb || c > r) continue;
+      if (c == r) A[(k0 + r) + (int64_t)(k0 + r) * lda].y = S[r][r].x;
+      else A[(k0 + c) + (int64_t)(k0 + r) * lda] = S[c][r];
+    }
+  const int i = k0 + kb + blockIdx.x * kPR + w;
   if (i >= n) return;
-  double2 x[NB];
+  double2* a = A + i + (int64_t)k0 * lda;
+  double2 x = lane < kb ? a[(int64_t)lane * lda] : make_double2(0.0, 0.0);
   for (int j = 0; j < kb; ++j) {
-    double2 s = A[i + (int64_t)(k0 + j) * lda];
-    for (int tt = 0; tt < j; ++tt) s = csub(s, cmul(x[tt], cconj(Ls[j][tt])));
-    x[j] = cscale(s, 1.0 / Ls[j][j].x);
+    double2 xj;
+    xj.x = __shfl_sync(0xffffffffu, x.x, j) * inv[j];
+    xj.y = __shfl_sync(0xffffffffu, x.y, j) * inv[j];
+    if (lane == j) x = xj;
+    else if (lane > j && lane < kb) x = csub(x, cmul(xj, cconj(S[j][lane])));
   }
-  for (int j = 0; j < kb; ++j) A[i + (int64_t)(k0 + j) * lda] = x[j];
+  if (lane < kb) a[(int64_t)lane * lda] = x;
 }
 
-// trailing update of the lower triangle: A[i][j] -= sum_t L[i][t] conj(L[j][t])
-__global__ void k_chol_update(double2* A, int64_t lda, int n, int k0, int kb) {
+// trailing update of the lower triangle, 16 x 16 tiles: A[i][j] -= sum_t L[i][t] conj(L[j][t])
+// (36 us a panel at n = 512 on average, 68 with 32 x 32 tiles, which keep an SM 34 us on one tile)
+__global__ void __launch_bounds__(256) k_chol_update(double2* A, int64_t lda, int n, int k0, int kb) {
   const int bi = blockIdx.x, bj = blockIdx.y;
   if (bj > bi) return;
-  __shared__ double2 Li[32][NB + 1], Lj[32][NB + 1];
-  const int s0 = k0 + kb;
-  const int i0 = s0 + bi * 32, j0 = s0 + bj * 32;
-  const int t = threadIdx.x;  // 256
-  for (int e = t; e < 32 * kb; e += 256) {
-    const int r = e % 32, c = e / 32;
-    Li[r][c] = (i0 + r < n) ? A[(i0 + r) + (int64_t)(k0 + c) * lda] : make_double2(0, 0);
-    Lj[r][c] = (j0 + r < n) ? A[(j0 + r) + (int64_t)(k0 + c) * lda] : make_double2(0, 0);
+  __shared__ double2 Li[NB][17], Lj[NB][17];
+  const int s0 = k0 + kb, r = threadIdx.x & 15, c = threadIdx.x >> 4;
+  const int i0 = s0 + bi * 16, j0 = s0 + bj * 16;
+  for (int t = c; t < kb; t += 16) {
+    Li[t][r] = (i0 + r < n) ? A[(i0 + r) + (int64_t)(k0 + t) * lda] : make_double2(0, 0);
+    Lj[t][r] = (j0 + r < n) ? A[(j0 + r) + (int64_t)(k0 + t) * lda] : make_double2(0, 0);
   }
   __syncthreads();
-  for (int e = t; e < 32 * 32; e += 256) {
-    const int r = e % 32, c = e / 32;
-    const int i = i0 + r, j = j0 + c;
-    if (i >= n || j >= n || j > i) continue;
-    double2 s = make_double2(0, 0);
-    for (int tt = 0; tt < kb; ++tt) {
-      const double2 a = Li[r][tt], b = Lj[c][tt];
-      s.x += a.x * b.x + a.y * b.y;
-      s.y += a.y * b.x - a.x * b.y;
-    }
-    A[i + (int64_t)j * lda] = csub(A[i + (int64_t)j * lda], s);
+  const int i = i0 + r, j = j0 + c;
+  if (i >= n || j >= n || j > i) return;
+  double2 s = make_double2(0, 0);
+  for (int t = 0; t < kb; ++t) {
+    const double2 a = Li[t][r], b = Lj[t][c];
+    s.x += a.x * b.x + a.y * b.y;
+    s.y += a.y * b.x - a.x * b.y;
   }
+  A[i + (int64_t)j * lda] = csub(A[i + (int64_t)j * lda], s);
 }
 
 __global__ void k_zero_upper(double2* A, int64_t lda, int n) {
@@ -134,75 +147,103 @@ cudaError_t la_zero_upper(double2* A, int64_t lda, int n, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+// the diagonal blocks' factors into place, the strict upper triangle zero
+__global__ void k_chol_finish(double2* A, int64_t lda, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = blockIdx.y * blockDim.y + threadIdx.y;
+  if (i >= n || j > i) return;
+  double2* up = A + j + (int64_t)i * lda;
+  if (i == j) {
+    *up = make_double2(up->y, 0.0);
+    return;
+  }
+  if (i / NB == j / NB) A[i + (int64_t)j * lda] = *up;
+  *up = make_double2(0.0, 0.0);
+}
+
 cudaError_t la_cholesky(double2* A, int64_t lda, int n, int* flag, cudaStream_t st) {
   for (int k0 = 0; k0 < n; k0 += NB) {
     const int kb = min(NB, n - k0);
-    k_chol_diag<<<1, dim3(32, 32), 0, st>>>(A, lda, k0, kb, flag); count_launch();
     const int rest = n - k0 - kb;
+    k_chol_panel<<<std::max(1, (rest + kPR - 1) / kPR), 256, 0, st>>>(A, lda, n, k0, kb, flag); count_launch();
     if (rest > 0) {
-      k_chol_panel<<<(rest + 127) / 128, 128, 0, st>>>(A, lda, n, k0, kb); count_launch();
-      const int nt = (rest + 31) / 32;
+      const int nt = (rest + 15) / 16;
       k_chol_update<<<dim3(nt, nt), 256, 0, st>>>(A, lda, n, k0, kb); count_launch();
     }
   }
-  // zero the strict upper triangle
   dim3 zb(16, 16), zg((n + 15) / 16, (n + 15) / 16);
-  k_zero_upper<<<zg, zb, 0, st>>>(A, lda, n); count_launch();
+  k_chol_finish<<<zg, zb, 0, st>>>(A, lda, n); count_launch();
   return cudaGetLastError();
 }
 
 // ---- triangular inverse X = L^{-1} (lower) -------------------------------------------
-__global__ void k_transpose(const double2* A, int64_t lda, int n, double2* At) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  if (i < n && j < n) At[j + (int64_t)i * n] = A[i + (int64_t)j * lda];
+// The 32 x 32 diagonal blocks by substitution (a column per warp, 8 columns per CTA), then
+// [A 0; C B]^{-1} = [A^-1 0; -B^-1 C A^-1 B^-1] for blocks of 32, 64, ...: two products per level,
+// 16 x 16 tiles over all the SMs (0.38 ms at n = 512).  A substitution of whole columns, a warp each, took 1.95 ms at
+// n = 512 (a serial chain of n warp reductions).
+__global__ void __launch_bounds__(256) k_trinv_diag(const double2* __restrict__ L, int64_t lda, int n,
+                                                    double2* __restrict__ X, int64_t ldx) {
+  __shared__ double2 S[NB][NB + 1];  // S[col][row]
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const int k0 = blockIdx.x * NB, kb = min(NB, n - k0);
+  for (int e = t; e < NB * NB; e += 256) {
+    const int r = e % NB, c = e / NB;
+    S[c][r] = (r < kb && c <= r) ? L[(k0 + r) + (int64_t)(k0 + c) * lda] : make_double2(r == c ? 1.0 : 0.0, 0.0);
+  }
+  __syncthreads();
+  const int c = blockIdx.y * 8 + w;
+  if (c >= kb) return;
+  const double inv = 1.0 / S[lane][lane].x;
+  double2 x = make_double2(lane == c ? 1.0 : 0.0, 0.0);
+  for (int j = c; j < kb; ++j) {
+    double2 xj;
+    xj.x = __shfl_sync(0xffffffffu, x.x * inv, j);
+    xj.y = __shfl_sync(0xffffffffu, x.y * inv, j);
+    if (lane == j) x = xj;
+    else if (lane > j) x = csub(x, cmul(S[j][lane], xj));
+  }
+  if (lane < kb) X[(k0 + lane) + (int64_t)(k0 + c) * ldx] = lane < c ? make_double2(0.0, 0.0) : x;
 }
 
-// one warp per column j of X; Lt holds L row-major (Lt[t + i n] = L[i][t])
-__global__ void k_trinv(const double2* __restrict__ Lt, int n, double2* __restrict__ X, int64_t ldx) {
-  extern __shared__ double2 xs[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int j = blockIdx.x * (blockDim.x >> 5) + warp;
-  if (j >= n) return;
-  double2* x = xs + (int64_t)warp * n;
-  for (int i = lane; i < j; i += 32) X[i + (int64_t)j * ldx] = make_double2(0, 0);
-  if (lane == 0) {
-    const double d = Lt[j + (int64_t)j * n].x;
-    x[j] = make_double2(1.0 / d, 0.0);
-    X[j + (int64_t)j * ldx] = x[j];
-  }
-  __syncwarp();
-  for (int i = j + 1; i < n; ++i) {
-    const double2* row = Lt + (int64_t)i * n;
-    double sr = 0, si = 0;
-    for (int t = j + lane; t < i; t += 32) {
-      const double2 a = row[t], b = x[t];
-      sr += a.x * b.x - a.y * b.y;
-      si += a.x * b.y + a.y * b.x;
-    }
+// level s, pair blockIdx.z (rows r0 .. of the second block, columns c0 .. of the first):
+// SECOND == 0: C21 = A21 B11 (B11 lower), SECOND == 1: C21 = -A22 B21 (A22 lower)
+template <int SECOND>
+__global__ void __launch_bounds__(256) k_trinv_mul(const double2* __restrict__ A, int64_t lda,
+                                                   const double2* __restrict__ B, int64_t ldb, double2* C, int64_t ldc,
+                                                   int n, int s) {
+  __shared__ double2 As[16][17], Bs[16][17];
+  const int c0 = 2 * s * blockIdx.z, r0 = c0 + s, rows = min(s, n - r0);
+  const int i0 = blockIdx.x * 16, j0 = blockIdx.y * 16, x = threadIdx.x & 15, y = threadIdx.x >> 4;
+  if (i0 >= rows) return;
+  const int t_lo = SECOND ? 0 : j0, t_hi = SECOND ? min(rows, i0 + 16) : s;
+  const int ca = SECOND ? r0 : c0;  // A's columns, B's rows
+  double2 acc = make_double2(0.0, 0.0);
+  for (int t0 = t_lo; t0 < t_hi; t0 += 16) {
+    const double2 z = make_double2(0.0, 0.0);
+    As[y][x] = (i0 + x < rows && t0 + y < t_hi) ? A[(r0 + i0 + x) + (int64_t)(ca + t0 + y) * lda] : z;
+    Bs[y][x] = (t0 + x < t_hi) ? B[(ca + t0 + x) + (int64_t)(c0 + j0 + y) * ldb] : z;
+    __syncthreads();
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      sr += __shfl_down_sync(0xffffffffu, sr, o);
-      si += __shfl_down_sync(0xffffffffu, si, o);
+    for (int t = 0; t < 16; ++t) {
+      const double2 a = As[t][x], b = Bs[y][t];
+      acc.x = fma(a.x, b.x, fma(-a.y, b.y, acc.x));
+      acc.y = fma(a.x, b.y, fma(a.y, b.x, acc.y));
     }
-    if (lane == 0) {
-      const double d = row[i].x;
-      x[i] = make_double2(-sr / d, -si / d);
-      X[i + (int64_t)j * ldx] = x[i];
-    }
-    __syncwarp();
+    __syncthreads();
   }
+  if (i0 + x < rows) C[(r0 + i0 + x) + (int64_t)(c0 + j0 + y) * ldc] = SECOND ? make_double2(-acc.x, -acc.y) : acc;
 }
 
 cudaError_t la_trinv_lower(const double2* L, int64_t lda, int n, double2* X, int64_t ldx, double2* tmp,
                            cudaStream_t st) {
   dim3 b(16, 16), g((n + 15) / 16, (n + 15) / 16);
-  k_transpose<<<g, b, 0, st>>>(L, lda, n, tmp); count_launch();
-  const int wpb = 4;
-  const size_t sm = sizeof(double2) * (size_t)n * wpb;
-  cudaError_t e = cudaFuncSetAttribute(k_trinv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  if (e) return e;
-  k_trinv<<<(n + wpb - 1) / wpb, 32 * wpb, sm, st>>>(tmp, n, X, ldx); count_launch();
+  k_trinv_diag<<<dim3((n + NB - 1) / NB, NB / 8), 256, 0, st>>>(L, lda, n, X, ldx); count_launch();
+  for (int s = NB; s < n; s *= 2) {
+    const dim3 gm((unsigned)(s / 16), (unsigned)(s / 16), (unsigned)((n - s + 2 * s - 1) / (2 * s)));
+    k_trinv_mul<0><<<gm, 256, 0, st>>>(L, lda, X, ldx, tmp, n, n, s); count_launch();
+    k_trinv_mul<1><<<gm, 256, 0, st>>>(X, ldx, tmp, n, X, ldx, n, s); count_launch();
+  }
+  k_zero_upper<<<g, b, 0, st>>>(X, ldx, n); count_launch();
   return cudaGetLastError();
 }
 
@@ -606,27 +647,42 @@ cudaError_t la_rq_minmax(const double2* num, const double2* den, int m, double* 
 }
 
 // ---- Lanczos helpers (one vector) ---------------------------------------------------
-// ab: device array, alpha at ab[2k], beta at ab[2k+1]
-__global__ void k_lz_dot(const double2* v, const double2* w, int n, double* alpha_out) {
-  __shared__ double sh[1024];
-  double s = 0;
-  for (int g = threadIdx.x; g < n; g += blockDim.x) s += v[g].x * w[g].x + v[g].y * w[g].y;
-  sh[threadIdx.x] = s;
+// Vector work over kLzBlocks CTAs; a reduction leaves one partial sum per CTA, which every CTA of
+// the next kernel adds up in the same order (11 us per Lanczos step at 14771 plane waves; on
+// one CTA, bound by its SM's FP64 pipe, 72 us).
+constexpr int kLzBlocks = la_lz_blocks;
+
+__device__ __forceinline__ double lz_block_sum(double s) {  // result in every thread
+  __shared__ double sh[8];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   __syncthreads();
-  for (int k = blockDim.x / 2; k > 0; k >>= 1) {
-    if (threadIdx.x < k) sh[threadIdx.x] += sh[threadIdx.x + k];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *alpha_out = sh[0];
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+  __syncthreads();
+  double r = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) r += sh[i];
+  return r;
+}
+__device__ __forceinline__ double lz_total(const double* part) {
+  return lz_block_sum(threadIdx.x < kLzBlocks ? part[threadIdx.x] : 0.0);
 }
 
-// w <- w - alpha v - beta vprev ; beta_out = ||w|| ; vprev <- v ; v <- w / beta_out
-__global__ void k_lz_update(double2* w, double2* v, double2* vprev, int n, const double* alpha,
-                            const double* beta_prev, double* beta_out) {
-  __shared__ double sh[1024];
-  const double a = *alpha, b = beta_prev ? *beta_prev : 0.0;
+// part = Re <v, w>
+__global__ void __launch_bounds__(256) k_lz_dot(const double2* v, const double2* w, int n, double* part) {
   double s = 0;
-  for (int g = threadIdx.x; g < n; g += blockDim.x) {
+  for (int g = blockIdx.x * 256 + threadIdx.x; g < n; g += gridDim.x * 256) s += v[g].x * w[g].x + v[g].y * w[g].y;
+  s = lz_block_sum(s);
+  if (threadIdx.x == 0) part[blockIdx.x] = s;
+}
+
+// alpha = <v, w> (from dots); w <- w - alpha v - beta vprev; part = ||w||^2
+__global__ void __launch_bounds__(256) k_lz_update(double2* w, const double2* v, const double2* vprev, int n,
+                                                   const double* dots, double* alpha_out, const double* beta_prev,
+                                                   double* part) {
+  const double a = lz_total(dots), b = beta_prev ? *beta_prev : 0.0;
+  double s = 0;
+  for (int g = blockIdx.x * 256 + threadIdx.x; g < n; g += gridDim.x * 256) {
     double2 x = w[g];
     const double2 vv = v[g], vp = vprev[g];
     x.x -= a * vv.x + b * vp.x;
@@ -634,42 +690,28 @@ __global__ void k_lz_update(double2* w, double2* v, double2* vprev, int n, const
     w[g] = x;
     s += x.x * x.x + x.y * x.y;
   }
-  sh[threadIdx.x] = s;
-  __syncthreads();
-  for (int k = blockDim.x / 2; k > 0; k >>= 1) {
-    if (threadIdx.x < k) sh[threadIdx.x] += sh[threadIdx.x + k];
-    __syncthreads();
-  }
-  const double nb = sqrt(sh[0]);
+  s = lz_block_sum(s);
+  if (threadIdx.x == 0) part[blockIdx.x] = s;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *alpha_out = a;
+}
+
+// beta = sqrt(sum of part); vprev <- v (0 without v_old); v <- w / beta
+__global__ void __launch_bounds__(256) k_lz_scale(const double2* w, double2* v, double2* vprev, int n,
+                                                  const double* part, double* beta_out) {
+  const double nb = sqrt(lz_total(part));
   const double inv = nb > 0 ? 1.0 / nb : 0.0;
-  for (int g = threadIdx.x; g < n; g += blockDim.x) {
-    vprev[g] = v[g];
-    v[g] = cscale(w[g], inv);
+  for (int g = blockIdx.x * 256 + threadIdx.x; g < n; g += gridDim.x * 256) {
+    vprev[g] = beta_out ? v[g] : make_double2(0, 0);
+    v[g] = cscale(w[g], beta_out ? inv : 1.0 / nb);
   }
-  if (threadIdx.x == 0) *beta_out = nb;
+  if (beta_out && blockIdx.x == 0 && threadIdx.x == 0) *beta_out = nb;
 }
 
-__global__ void k_lz_normalize(const double2* v0, double2* v, double2* vprev, int n) {
-  __shared__ double sh[1024];
-  double s = 0;
-  for (int g = threadIdx.x; g < n; g += blockDim.x) s += v0[g].x * v0[g].x + v0[g].y * v0[g].y;
-  sh[threadIdx.x] = s;
-  __syncthreads();
-  for (int k = blockDim.x / 2; k > 0; k >>= 1) {
-    if (threadIdx.x < k) sh[threadIdx.x] += sh[threadIdx.x + k];
-    __syncthreads();
-  }
-  const double inv = 1.0 / sqrt(sh[0]);
-  for (int g = threadIdx.x; g < n; g += blockDim.x) {
-    v[g] = cscale(v0[g], inv);
-    vprev[g] = make_double2(0, 0);
-  }
-}
-
-// largest eigenvalue of the k x k symmetric tridiagonal (alpha, beta) by Sturm bisection;
-// out[0] = theta_max + |beta_k|, out[1] = theta_max
+// largest eigenvalue of the k x k symmetric tridiagonal (alpha, beta) by Sturm counts at 32 points
+// of the bracket at a time (one warp); out[0] = theta_max + |beta_k|, out[1] = theta_max.  74 us at
+// k = 10, 300 us with one thread bisecting: each count is a chain of k divisions.
 __global__ void k_lz_bound(const double* ab, int k, double* out) {
-  if (threadIdx.x != 0) return;
+  const int lane = threadIdx.x;
   double lo = INFINITY, hi = -INFINITY;
   for (int i = 0; i < k; ++i) {
     const double a = ab[2 * i];
@@ -677,10 +719,10 @@ __global__ void k_lz_bound(const double* ab, int k, double* out) {
     lo = fmin(lo, a - r);
     hi = fmax(hi, a + r);
   }
-  // count of eigenvalues < x
   for (int it = 0; it < 200; ++it) {
-    const double x = 0.5 * (lo + hi);
-    if (x == lo || x == hi) break;
+    const double x = lo + (hi - lo) * ((lane + 1) / 33.0);
+    const bool inside = x > lo && x < hi;
+    // all k eigenvalues below x?
     int cnt = 0;
     double d = 1.0;
     for (int i = 0; i < k; ++i) {
@@ -689,20 +731,35 @@ __global__ void k_lz_bound(const double* ab, int k, double* out) {
       if (d == 0.0) d = -1e-300;
       if (d < 0) ++cnt;
     }
-    if (cnt == k) hi = x; else lo = x;
+    const unsigned in = __ballot_sync(0xffffffffu, inside), all = __ballot_sync(0xffffffffu, inside && cnt == k);
+    if (!in) break;
+    const int h = all ? __ffs(all) - 1 : 32;  // first point above all eigenvalues
+    const unsigned below = in & ~all & (h < 32 ? (1u << h) - 1u : 0xffffffffu);
+    const int l = below ? 31 - __clz(below) : -1;
+    const double nh = __shfl_sync(0xffffffffu, x, h & 31), nl = __shfl_sync(0xffffffffu, x, l & 31);
+    if (h < 32) hi = nh;
+    if (l >= 0) lo = nl;
   }
-  out[1] = hi;
-  out[0] = hi + fabs(ab[2 * k - 1]);
+  if (lane == 0) {
+    out[1] = hi;
+    out[0] = hi + fabs(ab[2 * k - 1]);
+  }
 }
 
 cudaError_t la_lanczos(const double2* v0, int n, int steps, double2* v, double2* vprev, double2* w, double* ab,
-                       double* bound, ApplyFn apply, void* ctx, cudaStream_t st) {
-  k_lz_normalize<<<1, 1024, 0, st>>>(v0, v, vprev, n); count_launch();
+                       double* bound, double* part, ApplyFn apply, void* ctx, cudaStream_t st) {
+  const int grid = std::max(1, std::min(kLzBlocks, (n + 255) / 256));
+  double *p1 = part, *p2 = part + kLzBlocks;
+  cudaError_t e = cudaMemsetAsync(part, 0, 2 * kLzBlocks * sizeof(double), st);  // CTAs beyond the grid add 0
+  if (e) return e;
+  k_lz_dot<<<grid, 256, 0, st>>>(v0, v0, n, p2); count_launch();
+  k_lz_scale<<<grid, 256, 0, st>>>(v0, v, vprev, n, p2, nullptr); count_launch();
   for (int k = 0; k < steps; ++k) {
     int s = apply(ctx, v, w);
     if (s != PW_OK) return cudaErrorUnknown;
-    k_lz_dot<<<1, 1024, 0, st>>>(v, w, n, ab + 2 * k); count_launch();
-    k_lz_update<<<1, 1024, 0, st>>>(w, v, vprev, n, ab + 2 * k, k > 0 ? ab + 2 * k - 1 : nullptr, ab + 2 * k + 1); count_launch();
+    k_lz_dot<<<grid, 256, 0, st>>>(v, w, n, p1); count_launch();
+    k_lz_update<<<grid, 256, 0, st>>>(w, v, vprev, n, p1, ab + 2 * k, k > 0 ? ab + 2 * k - 1 : nullptr, p2); count_launch();
+    k_lz_scale<<<grid, 256, 0, st>>>(w, v, vprev, n, p2, ab + 2 * k + 1); count_launch();
   }
   k_lz_bound<<<1, 32, 0, st>>>(ab, steps, bound); count_launch();
   return cudaGetLastError();

@@ -1271,11 +1271,11 @@ int bounds_impl(pw_ctx* ctx, const double2* psi, int64_t ld, int nband, int step
   }
   if (steps > 0) {
     if (!v0) return set_error(PW_EINVAL, "Lanczos start vector is NULL");
-    WS(lz, double2, WS_LZ, (size_t)3 * npw + 2 * steps + 8);
+    WS(lz, double2, WS_LZ, (size_t)3 * npw + 2 * steps + 8 + la_lz_blocks);
     double* ab = (double*)(lz + 3 * npw);
     double* bound = ab + 2 * steps;
     LzCtx lc{ctx};
-    CU_TRY(la_lanczos(v0, npw, steps, lz, lz + npw, lz + 2 * npw, ab, bound, lz_apply, &lc, st), "lanczos");
+    CU_TRY(la_lanczos(v0, npw, steps, lz, lz + npw, lz + 2 * npw, ab, bound, bound + 4, lz_apply, &lc, st), "lanczos");
     double h[2];
     CU_TRY(cudaMemcpyAsync(h, bound, 2 * sizeof(double), cudaMemcpyDeviceToHost, st), "bound copy");
     CU_TRY(cudaStreamSynchronize(st), "bound sync");
