@@ -25,8 +25,10 @@
 #include <type_traits>
 #include <utility>
 
-#include "pw_internal.cuh"
 #include "fft_fixed.cuh"
+#include "fft_lines.cuh"
+#include "fft_radix.cuh"
+#include "pw_internal.cuh"
 
 namespace pw {
 
@@ -36,150 +38,6 @@ constexpr bool xf_twr(int xf) { return xf >= 3 && xf <= 10; }
 constexpr bool xf_multi(int xf) { return xf == 4 || xf == 6 || xf == 8 || xf == 10; }
 constexpr bool xf_swap(int xf) { return xf == 5 || xf == 6 || xf == 9 || xf == 10; }
 constexpr bool xf_staged(int xf) { return xf >= 7 && xf <= 10; }
-
-// ---- butterfly arithmetic ---------------------------------------------------------
-// complex64 sums, differences and real scalings use the paired FP32 instructions of
-// sm_100-class SMs (one add, multiply or fused multiply-add for both halves of a float2,
-// each half rounded to nearest as the scalar instruction would); complex128 keeps the
-// scalar forms.  The products by +-i swap the halves of an operand, which a paired
-// instruction cannot do in place, so they stay two scalar instructions (measured on the
-// 120^3 plane passes: 6% faster than paired with the swap; all-scalar butterflies are
-// slower still).  Every form rounds each result identically.
-__device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
-__device__ __forceinline__ double2 bf_add(double2 a, double2 b) { return cadd(a, b); }
-__device__ __forceinline__ float2 bf_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ double2 bf_sub(double2 a, double2 b) { return csub(a, b); }
-__device__ __forceinline__ float2 bf_sub(float2 a, float2 b) { return __ffma2_rn(b, f2(-1.f, -1.f), a); }
-__device__ __forceinline__ double2 bf_scale(double2 a, double s) { return cscale(a, s); }
-__device__ __forceinline__ float2 bf_scale(float2 a, float s) { return __fmul2_rn(a, f2(s, s)); }
-// a + s b
-__device__ __forceinline__ double2 bf_axpy(double2 a, double s, double2 b) {
-  return make_double2(fma(s, b.x, a.x), fma(s, b.y, a.y));
-}
-__device__ __forceinline__ float2 bf_axpy(float2 a, float s, float2 b) { return __ffma2_rn(b, f2(s, s), a); }
-// a + (S i) s b  and  a - (S i) s b
-template <int S> __device__ __forceinline__ double2 bf_add_muli(double2 a, double2 b, double s = 1.0) {
-  return make_double2(fma(-S * s, b.y, a.x), fma(S * s, b.x, a.y));
-}
-template <int S> __device__ __forceinline__ float2 bf_add_muli(float2 a, float2 b, float s = 1.f) {
-  return f2(__fmaf_rn(-S * s, b.y, a.x), __fmaf_rn(S * s, b.x, a.y));
-}
-template <int S> __device__ __forceinline__ double2 bf_sub_muli(double2 a, double2 b, double s = 1.0) {
-  return make_double2(fma(S * s, b.y, a.x), fma(-S * s, b.x, a.y));
-}
-template <int S> __device__ __forceinline__ float2 bf_sub_muli(float2 a, float2 b, float s = 1.f) {
-  return f2(__fmaf_rn(S * s, b.y, a.x), __fmaf_rn(-S * s, b.x, a.y));
-}
-
-// ---- small DFTs: y_m = sum_k x_k exp(S 2 pi i k m / R) -------------------------
-template <typename C, int S> __device__ __forceinline__ void dft2(C& a, C& b) {
-  C t = a; a = bf_add(t, b); b = bf_sub(t, b);
-}
-template <typename C, int S> __device__ __forceinline__ void dft4(C* x) {
-  C s02 = bf_add(x[0], x[2]), d02 = bf_sub(x[0], x[2]);
-  C s13 = bf_add(x[1], x[3]), d13 = bf_sub(x[1], x[3]);
-  x[0] = bf_add(s02, s13); x[2] = bf_sub(s02, s13);
-  x[1] = bf_add_muli<S>(d02, d13); x[3] = bf_sub_muli<S>(d02, d13);
-}
-template <typename C, int S> __device__ __forceinline__ void dft8(C* x) {
-  using R = decltype(C{}.x);
-  const R h = (R)0.70710678118654752440084436210485;  // cos(pi/4)
-  C e[4] = {x[0], x[2], x[4], x[6]};
-  C o[4] = {x[1], x[3], x[5], x[7]};
-  dft4<C, S>(e); dft4<C, S>(o);
-  // o[m] *= w8^m, w8 = exp(S i pi/4): w8 = h (1 + S i), w8^3 = h (-1 + S i)
-  const C o1 = bf_scale(bf_add_muli<S>(o[1], o[1]), h);
-  const C o3 = bf_scale(bf_sub_muli<S>(o[3], o[3]), -h);
-  x[0] = bf_add(e[0], o[0]); x[4] = bf_sub(e[0], o[0]);
-  x[1] = bf_add(e[1], o1); x[5] = bf_sub(e[1], o1);
-  x[2] = bf_add_muli<S>(e[2], o[2]); x[6] = bf_sub_muli<S>(e[2], o[2]);
-  x[3] = bf_add(e[3], o3); x[7] = bf_sub(e[3], o3);
-}
-template <typename C, int S> __device__ __forceinline__ void dft3(C* x) {
-  using R = decltype(C{}.x);
-  const R s3 = (R)0.86602540378443864676372317075294;  // sin(pi/3)
-  C t = bf_add(x[1], x[2]);
-  C d = bf_sub(x[1], x[2]);
-  C m = bf_axpy(x[0], (R)-0.5, t);
-  x[0] = bf_add(x[0], t);
-  x[1] = bf_add_muli<S>(m, d, s3);
-  x[2] = bf_sub_muli<S>(m, d, s3);
-}
-template <typename C, int S> __device__ __forceinline__ void dft5(C* x) {
-  using R = decltype(C{}.x);
-  const R c1 = (R)0.30901699437494742410229341718282;   // cos(2pi/5)
-  const R c2 = (R)-0.80901699437494742410229341718282;  // cos(4pi/5)
-  const R s1 = (R)0.95105651629515357211643933337938;   // sin(2pi/5)
-  const R s2 = (R)0.58778525229247312916870595463907;   // sin(4pi/5)
-  C t1 = bf_add(x[1], x[4]), t2 = bf_add(x[2], x[3]);
-  C d1 = bf_sub(x[1], x[4]), d2 = bf_sub(x[2], x[3]);
-  C a1 = bf_add(x[0], bf_axpy(bf_scale(t1, c1), c2, t2));
-  C a2 = bf_add(x[0], bf_axpy(bf_scale(t1, c2), c1, t2));
-  C u1 = bf_axpy(bf_scale(d1, s1), s2, d2);    // b1 = (S i) u1
-  C u2 = bf_axpy(bf_scale(d1, s2), -s1, d2);   // b2 = (S i) u2
-  x[0] = bf_add(x[0], bf_add(t1, t2));
-  x[1] = bf_add_muli<S>(a1, u1); x[4] = bf_sub_muli<S>(a1, u1);
-  x[2] = bf_add_muli<S>(a2, u2); x[3] = bf_sub_muli<S>(a2, u2);
-}
-// exp(-2 pi i m / R) for the composite in-register radices, filled by fft_set_constants
-// (host cos/sin in double).  Offsets: R=6: 0, 9: 6, 10: 15, 12: 25, 15: 37, 16: 52.
-__constant__ double2 c_wtab64[68];
-__constant__ float2 c_wtab32[68];
-template <int R> struct WOff;
-template <> struct WOff<6> { static constexpr int v = 0; };
-template <> struct WOff<9> { static constexpr int v = 6; };
-template <> struct WOff<10> { static constexpr int v = 15; };
-template <> struct WOff<12> { static constexpr int v = 25; };
-template <> struct WOff<15> { static constexpr int v = 37; };
-template <> struct WOff<16> { static constexpr int v = 52; };
-
-template <typename C, int S, int R> __device__ __forceinline__ C wconst(int m) {
-  C w;
-  if constexpr (sizeof(C) == 16) { const double2 t = c_wtab64[WOff<R>::v + m]; w.x = t.x; w.y = t.y; }
-  else { const float2 t = c_wtab32[WOff<R>::v + m]; w.x = t.x; w.y = t.y; }
-  if (S > 0) w.y = -w.y;
-  return w;
-}
-
-template <typename C, int S, int R> __device__ __forceinline__ void dftR(C* x);
-
-// R = R1 R2 in registers: R2 DFTs of length R1 (stride R2), constant twiddles w_R^{b k1},
-// R1 DFTs of length R2; natural-order output X[k1 + R1 k2].
-template <typename C, int S, int R, int R1, int R2> __device__ __forceinline__ void dft_comp(C* x) {
-  C t[R];
-#pragma unroll
-  for (int b = 0; b < R2; ++b) {
-    C u[R1];
-#pragma unroll
-    for (int a = 0; a < R1; ++a) u[a] = x[b + R2 * a];
-    dftR<C, S, R1>(u);
-#pragma unroll
-    for (int k1 = 0; k1 < R1; ++k1) t[b + R2 * k1] = (b * k1 == 0) ? u[k1] : cmul(u[k1], wconst<C, S, R>(b * k1));
-  }
-#pragma unroll
-  for (int k1 = 0; k1 < R1; ++k1) {
-    C v[R2];
-#pragma unroll
-    for (int b = 0; b < R2; ++b) v[b] = t[b + R2 * k1];
-    dftR<C, S, R2>(v);
-#pragma unroll
-    for (int k2 = 0; k2 < R2; ++k2) x[k1 + R1 * k2] = v[k2];
-  }
-}
-
-template <typename C, int S, int R> __device__ __forceinline__ void dftR(C* x) {
-  if constexpr (R == 2) dft2<C, S>(x[0], x[1]);
-  else if constexpr (R == 3) dft3<C, S>(x);
-  else if constexpr (R == 4) dft4<C, S>(x);
-  else if constexpr (R == 5) dft5<C, S>(x);
-  else if constexpr (R == 8) dft8<C, S>(x);
-  else if constexpr (R == 6) dft_comp<C, S, 6, 3, 2>(x);
-  else if constexpr (R == 9) dft_comp<C, S, 9, 3, 3>(x);
-  else if constexpr (R == 10) dft_comp<C, S, 10, 5, 2>(x);
-  else if constexpr (R == 12) dft_comp<C, S, 12, 4, 3>(x);
-  else if constexpr (R == 15) dft_comp<C, S, 15, 5, 3>(x);
-  else dft_comp<C, S, 16, 4, 4>(x);
-}
 
 // one radix-R stage over `nlines` lines (line stride ls, element stride es)
 template <typename C, int S, bool DIT, bool LINE_FAST, int R>
@@ -2935,22 +2793,6 @@ static cudaError_t plane_tpl(int which, const cplx<T>* psi, int64_t ldpsi, cplx<
 }
 
 // ---- launchers ------------------------------------------------------------------
-cudaError_t fft_set_constants() {
-  const int Rs[6] = {6, 9, 10, 12, 15, 16};
-  double2 t64[68];
-  float2 t32[68];
-  int o = 0;
-  for (int r : Rs)
-    for (int m = 0; m < r; ++m, ++o) {
-      const double ang = -2.0 * 3.14159265358979323846264338327950288 * (double)m / (double)r;
-      t64[o] = make_double2(cos(ang), sin(ang));
-      t32[o] = make_float2((float)t64[o].x, (float)t64[o].y);
-    }
-  cudaError_t e = cudaMemcpyToSymbol(c_wtab64, t64, sizeof(t64));
-  if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_wtab32, t32, sizeof(t32));
-  return e;
-}
-
 static int pick_cz(int n3) { return n3 < 16 ? n3 : 16; }
 
 template <typename T>
@@ -3007,6 +2849,8 @@ cudaError_t launch_local_apply(const FftPlan& plan, const cplx<T>* tw, const Sph
   const bool tpl = pf == 1, pwg = pf == 2 || pf == 6, prs = pf == 3, pmix = pf == 4 || pf == 5;
   const bool ppers = pf == 5 || pf == 6, ipers = pf == 6;
   const bool xtw = xf == 2, xtwr = xf_twr(xf);
+  // boxes without a specialised kernel: the kernels for any two-stage plan, else the block-wide ones
+  const bool lines = fl::covers(plan);
   for (int b0 = 0; b0 < nband; b0 += band_batch) {
     const int nb = min(band_batch, nband - b0);
     prof_begin(prof, PW_PROF_PLANE_INV);
@@ -3020,6 +2864,12 @@ cudaError_t launch_local_apply(const FftPlan& plan, const cplx<T>* tw, const Sph
     if (e == cudaErrorNotSupported) {
       (void)cudaGetLastError();
       e = plane_lg<T>(0, psi + b0 * ldpsi, ldpsi, hb, hb_bs, sp, plan, tw, kin, nullptr, 0, nb, st);
+    }
+    if constexpr (std::is_same<T, float>::value) {
+      if (e == cudaErrorNotSupported && lines) {
+        (void)cudaGetLastError();
+        e = fl::inverse_planes(plan, tw, sp, psi + b0 * ldpsi, ldpsi, hb, hb_bs, nb, st);
+      }
     }
     if (e == cudaErrorNotSupported) {
       (void)cudaGetLastError();
@@ -3044,6 +2894,12 @@ cudaError_t launch_local_apply(const FftPlan& plan, const cplx<T>* tw, const Sph
       (void)cudaGetLastError();
       e = xline_lg<T>(hb, hb_bs, vperm, sp, plan, tw, nb, st);
     }
+    if constexpr (std::is_same<T, float>::value) {
+      if (e == cudaErrorNotSupported && lines) {
+        (void)cudaGetLastError();
+        e = fl::xlines(plan, tw, sp, vperm, hb, hb_bs, nb, st);
+      }
+    }
     if (e == cudaErrorNotSupported) {
       (void)cudaGetLastError();
       k_xline<T><<<dim3((nyz + lyz - 1) / lyz, nb), kThreads, sm2, st>>>(hb, hb_bs, vperm, sp, plan, tw, lyz); count_launch();
@@ -3065,6 +2921,13 @@ cudaError_t launch_local_apply(const FftPlan& plan, const cplx<T>* tw, const Sph
       (void)cudaGetLastError();
       e = plane_lg<T>(1, psi + b0 * ldpsi, ldpsi, hb, hb_bs, sp, plan, tw, kin, out + b0 * ldout, ldout, nb, st);
     }
+    if constexpr (std::is_same<T, float>::value) {
+      if (e == cudaErrorNotSupported && lines) {
+        (void)cudaGetLastError();
+        e = fl::forward_planes(plan, tw, sp, kin, hb, hb_bs, psi + b0 * ldpsi, ldpsi, out + b0 * ldout, ldout, nb, st,
+                               nullptr);
+      }
+    }
     if (e == cudaErrorNotSupported) {
       (void)cudaGetLastError();
       k_plane_fwd<T><<<dim3(sp.nplane, nb), kThreads, sm1, st>>>(hb, hb_bs, sp, plan, tw, cz, kin,
@@ -3082,11 +2945,16 @@ static bool plane_rs_covers(const FftPlan& plan) {
   return (n2 == 64 && n3 == 64) || (n2 == 72 && n3 == 90) || (n2 == 96 && n3 == 96) || (n2 == 120 && n3 == 120);
 }
 
+// boxes with line-group plane kernels: faster there than the kernels for any two-stage plan
+static bool plane_lg_covers(const FftPlan& plan) {
+  return plane_wg_covers(plan);  // the same boxes
+}
+
 bool local_apply_rec_supported(const FftPlan& plan, const ::pw_ctx* prof) {
   if (!prof) return false;
   const int pf = prof->fft_variant[0] / kFormStride;
   return ((pf == 2 || pf == 6) && plane_wg_covers(plan)) || (pf == 3 && plane_rs_covers(plan)) ||
-         ((pf == 4 || pf == 5) && plane_wg_covers(plan) && plane_rs_covers(plan));
+         ((pf == 4 || pf == 5) && plane_wg_covers(plan) && plane_rs_covers(plan)) || (pf >= 2 && fl::covers(plan) && !plane_lg_covers(plan));
 }
 
 cudaError_t launch_local_apply_rec(const FftPlan& plan, const float2* tw, const SphereDev& sp, const float* vperm,
@@ -3116,6 +2984,10 @@ cudaError_t launch_local_apply_rec(const FftPlan& plan, const float2* tw, const 
     e = inv_rs ? plane_rs<T>(0, psi + b0 * ldpsi, ldpsi, hb, hb_bs, sp, plan, tw, kin, nullptr, 0, nb, st, nullptr)
                : plane_wg<T>(0, psi + b0 * ldpsi, ldpsi, hb, hb_bs, sp, plan, tw, kin, nullptr, 0, nb, st, nullptr,
                              inv_pers);
+    if (e == cudaErrorNotSupported) {
+      (void)cudaGetLastError();
+      e = fl::inverse_planes(plan, tw, sp, psi + b0 * ldpsi, ldpsi, hb, hb_bs, nb, st);
+    }
     if (e) return e;
     prof_end(prof, PW_PROF_PLANE_INV);
     prof_begin(prof, PW_PROF_XLINE);
@@ -3128,6 +3000,10 @@ cudaError_t launch_local_apply_rec(const FftPlan& plan, const float2* tw, const 
     if (e == cudaErrorNotSupported) {
       (void)cudaGetLastError();
       e = xline_lg<T>(hb, hb_bs, vperm, sp, plan, tw, nb, st);
+    }
+    if (e == cudaErrorNotSupported && fl::covers(plan)) {
+      (void)cudaGetLastError();
+      e = fl::xlines(plan, tw, sp, vperm, hb, hb_bs, nb, st);
     }
     if (e == cudaErrorNotSupported) {
       (void)cudaGetLastError();
@@ -3146,6 +3022,11 @@ cudaError_t launch_local_apply_rec(const FftPlan& plan, const float2* tw, const 
                           &r)
             : plane_wg<T>(1, psi + b0 * ldpsi, ldpsi, hb, hb_bs, sp, plan, tw, kin, out + b0 * ldout, ldout, nb, st,
                           &r, fwd_pers);
+    if (e == cudaErrorNotSupported) {
+      (void)cudaGetLastError();
+      e = fl::forward_planes(plan, tw, sp, kin, hb, hb_bs, psi + b0 * ldpsi, ldpsi, out + b0 * ldout, ldout, nb, st,
+                             &r);
+    }
     if (e) return e;
     prof_end(prof, PW_PROF_PLANE_FWD);
   }

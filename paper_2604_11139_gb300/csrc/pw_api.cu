@@ -1440,7 +1440,6 @@ int create_impl(const pw_problem_desc* d, void* stream, pw_ctx** out) {
     PW_TRY(upload(ctx, &ctx->rho_perm[dd], r.data(), r.size()));
   }
   const cudaStream_t st = ctx->stream;
-  CU_TRY(fft_set_constants(), "FFT constants");
   // permuted potential, scaled by 1 / n1n2n3 (the forward DFT normalisation)
   const size_t ntot = (size_t)d->box[0] * d->box[1] * d->box[2];
   double* vraw;

@@ -200,17 +200,14 @@ struct Pass3Rec {
   int64_t split_ld, split_piece_stride;
   int pieces;
 };
-// H-apply local part with the fused recurrence of Pass3Rec (out = y_{k+1}); requires the
-// warp-group plane kernels for this box (plane form 2 of the context's complex64 variant),
-// else returns cudaErrorNotSupported before launching anything.
+// H-apply local part with the fused recurrence of Pass3Rec (out = y_{k+1}); requires a
+// plane form of the context's complex64 variant above 1 and a box that it or the kernels for any
+// two-stage plan (fft_lines.cu) cover, else returns cudaErrorNotSupported before launching anything.
 cudaError_t launch_local_apply_rec(const FftPlan& plan, const float2* tw, const SphereDev& sp, const float* vperm,
                                    const float* kin, const float2* psi, int64_t ldpsi, int nband, float2* out,
                                    int64_t ldout, float2* hb, int band_batch, cudaStream_t st, ::pw_ctx* prof,
                                    const Pass3Rec& rec);
 bool local_apply_rec_supported(const FftPlan& plan, const ::pw_ctx* prof);
-
-// fills the constant twiddles of the composite in-register radices on the current device
-cudaError_t fft_set_constants();
 
 template <typename T>
 cudaError_t launch_density(const FftPlan& plan, const cplx<T>* tw, const SphereDev& sp,
