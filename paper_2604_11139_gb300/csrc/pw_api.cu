@@ -249,9 +249,8 @@ Epi<T> epi(int mode, cplx<T>* out, int64_t ldo, T alpha = 1) {
   return e;
 }
 
-// Bands per FFT batch.  complex64: keep a batch's half-box planes near 48 MB so that
-// pass 1 -> pass 2 -> pass 3 hand the planes over through the 129 MB L2 instead of
-// HBM; complex128 (DFMA-bound) batches near 256 MB for fewer, larger launches.
+// Bands per FFT batch: half-box planes near fft_batch_bytes (complex64 384 MB, complex128 256 MB
+// unless tuned), a few large launches.
 int band_batch(const pw_ctx* ctx, int nband, size_t elem = 16) {
   const size_t per = (size_t)ctx->sp.nplane * ctx->n[1] * ctx->n[2] * elem;
   const size_t target = ctx->fft_batch_bytes[elem == 8 ? 0 : 1];

@@ -310,7 +310,9 @@ struct pw_ctx {
   bool poisoned = false;
   uint64_t ws_gen = 0;  // bumped whenever a workspace is (re)allocated (captured graphs check it)
   // tuning: bytes of half-box planes per FFT band batch (complex64, complex128); set by pw_autotune
-  size_t fft_batch_bytes[2] = {(size_t)48 << 20, (size_t)256 << 20};
+  // (complex64: large launches beat planes handed over in L2, 10-step filter of 128 bands on
+  // 72 x 72 x 90: 5.6 ms at 48 MB, 4.8 at 384 MB)
+  size_t fft_batch_bytes[2] = {(size_t)384 << 20, (size_t)256 << 20};
   // FFT pass kernel forms per precision, variant = xline form + 8 * plane form.  x-line
   // forms: 0 line groups of 1-8 threads with shared-memory twiddles, 1 one thread per line
   // with compile-time twiddles, 2 groups of warps per 32 lines (lane = line) with
@@ -318,10 +320,12 @@ struct pw_ctx {
   // 4 as 3 with several bands per CTA (V kept in registers); plane forms: 0 line groups,
   // 1 one thread per line, 2 groups of warps per 32 lines with table twiddles.  Forms other
   // than 0 cover two-stage plans in complex64 only (otherwise form 0 runs); set by pw_autotune
-  // FFT pass-kernel forms (complex64, complex128): complex128 defaults to the sphere-row +
+  // FFT pass-kernel forms (complex64, complex128): complex64 defaults to the staged multi-band
+  // x-lines (form 8) and plane form 3 with the recurrence in pass 3 (10-step filter of 128 bands on
+  // 72 x 72 x 90 with 48 MB batches: 5.5 ms, 10.0 on the line groups), complex128 to the sphere-row +
   // column-slice plane kernels (plane form 3), which fall back to line groups where they do
   // not apply (1.2x the line-group form on the 120^3 box)
-  int fft_variant[2] = {0, 3 * pw::kFormStride};
+  int fft_variant[2] = {8 + 3 * pw::kFormStride, 3 * pw::kFormStride};
   int last_sweeps = 0;  // Jacobi sweeps of the last Rayleigh-Ritz step
   // K splits of the mixed projection GEMM per column count, chosen by pw_autotune (columns ->
   // splits); other column counts use the whole-waves rule
