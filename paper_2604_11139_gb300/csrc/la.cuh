@@ -15,9 +15,12 @@ cudaError_t la_zero_upper(double2* A, int64_t lda, int n, cudaStream_t st);
 cudaError_t la_trinv_lower(const double2* L, int64_t lda, int n, double2* X, int64_t ldx, double2* tmp,
                            cudaStream_t st);
 // eigenpairs of Hermitian A (n x n, lda n; destroyed): eig ascending (device), U (n x n);
-// ws: 3 n*n + n + 2 complex; norms_dev: 2 doubles.  Synchronises the stream once per sweep.
+// ws: 3 n*n + n + 2 complex; norms_dev: 2 doubles.  Synchronises the stream once per sweep, and once
+// before the first with check_first (no sweep when A is diagonal to tol already).
 int la_jacobi_eigh(double2* A, int n, double2* U, double* eig, double2* ws, double* norms_dev,
-                   cudaStream_t st, int max_sweeps, double tol, int* sweeps_out);
+                   cudaStream_t st, int max_sweeps, double tol, bool check_first, int* sweeps_out);
+// K (n x n) <- I + the first-order correction of the eigenvectors of a nearly diagonal A
+cudaError_t la_eig_correction(const double2* A, int n, double2* K, cudaStream_t st);
 // FP32 Jacobi pre-rotation: V (n x n) <- the rotation that brings A (complex64, destroyed) to
 // off-diagonal norm below tol relative (or to the FP32 floor); ws: 2 n*n + n + 2 complex64
 int la_jacobi_rotate32(float2* A, int n, float2* V, float2* ws, double* norms_dev, cudaStream_t st, int max_sweeps,

@@ -49,6 +49,13 @@ cudaError_t la_herm_from_lower(double2* A, int64_t lda, int n, cudaStream_t st) 
 // ---- blocked Cholesky A = L L^dagger (lower, in place; strict upper part zeroed) ---
 constexpr int NB = 32;
 
+// s - a conj(b)
+__device__ __forceinline__ double2 csubmulc(double2 s, double2 a, double2 b) {
+  s.x = fma(-a.x, b.x, fma(-a.y, b.y, s.x));
+  s.y = fma(-a.y, b.x, fma(a.x, b.y, s.y));
+  return s;
+}
+
 // One panel: every CTA factors the 32 x 32 diagonal block for itself, in shared memory, and solves its kPR rows below, L21[i,:] = A21[i,:] L11^{-dagger}, one row per warp.
 // FP64 issues at 2 lanes per clock and SM, so the work is spread over as many SMs as it has rows /
 // 8, with the columns of a row over the lanes.  n = 512: 73 us a panel, the diagonal
@@ -75,7 +82,7 @@ __global__ void __launch_bounds__(256) k_chol_panel(double2* A, int64_t lda, int
       double d = S[j][j].x;
       const bool bad = !(d > 0.0) || !isfinite(d);
       if (bad) d = 1.0;
-      const double s = sqrt(d), i = 1.0 / s;
+      const double i = rsqrt(d), s = d * i;
       if (lane > j && lane < kb) S[j][lane] = cscale(S[j][lane], i);
       __syncwarp();
       if (lane == 0) {
@@ -87,7 +94,7 @@ __global__ void __launch_bounds__(256) k_chol_panel(double2* A, int64_t lda, int
     __syncthreads();
     // S[k][i] -= S[j][i] conj(S[j][k]) for j < k <= i: lane = row, the warps take the columns
     for (int k = j + 1 + w; k < kb; k += 8)
-      if (lane >= k && lane < kb) S[k][lane] = csub(S[k][lane], cmul(S[j][lane], cconj(S[j][k])));
+      if (lane >= k && lane < kb) S[k][lane] = csubmulc(S[k][lane], S[j][lane], S[j][k]);
     __syncthreads();
   }
   if (blockIdx.x == 0)
@@ -106,7 +113,7 @@ __global__ void __launch_bounds__(256) k_chol_panel(double2* A, int64_t lda, int
     xj.x = __shfl_sync(0xffffffffu, x.x, j) * inv[j];
     xj.y = __shfl_sync(0xffffffffu, x.y, j) * inv[j];
     if (lane == j) x = xj;
-    else if (lane > j && lane < kb) x = csub(x, cmul(xj, cconj(S[j][lane])));
+    else if (lane > j && lane < kb) x = csubmulc(x, xj, S[j][lane]);
   }
   if (lane < kb) a[(int64_t)lane * lda] = x;
 }
@@ -460,7 +467,7 @@ __global__ void k_offnorm(const C* A, int n, double* out) {
 // accumulated rotations in V; ws: 2 n*n + n + 2 complex of type C.  Returns the sweeps done.
 template <typename C>
 int jacobi_sweeps(C* A, int n, C* V, C* ws, double* norms_dev, cudaStream_t st, int max_sweeps, double tol,
-                  bool* converged, C** A_out, C** V_out) {
+                  bool check_first, bool* converged, C** A_out, C** V_out) {
   C* A2 = ws;
   C* V2 = ws + (int64_t)n * n;
   RotT<C>* rot = reinterpret_cast<RotT<C>*>(ws + 2 * (int64_t)n * n);
@@ -479,6 +486,17 @@ int jacobi_sweeps(C* A, int n, C* V, C* ws, double* norms_dev, cudaStream_t st, 
   // round in their own launch (recomputing them per CTA costs more FP64 time than the launch)
   constexpr bool kFused = sizeof(C) == 8;
   const int tpa = (npair + kJT - 1) / kJT, ta = tpa * tpa, tv = ((n + kJT - 1) / kJT) * tpa;
+  auto off_norm = [&]() -> int {  // h from the current matrix
+    cudaMemsetAsync(norms_dev, 0, 2 * sizeof(double), st);
+    k_offnorm<C><<<64, 256, 0, st>>>(Acur, n, norms_dev); count_launch();
+    cudaError_t e = cudaMemcpyAsync(h, norms_dev, 2 * sizeof(double), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    return e == cudaSuccess ? 0 : -1;
+  };
+  if (check_first && !conv) {
+    if (off_norm()) return -1;
+    conv = sqrt(h[0]) <= tol * sqrt(h[0] + h[1]);
+  }
   while (!conv && sweep < max_sweeps) {
     for (int t = 0; t < np - 1; ++t) {
       if (kFused) {
@@ -491,11 +509,7 @@ int jacobi_sweeps(C* A, int n, C* V, C* ws, double* norms_dev, cudaStream_t st, 
       x = Vcur; Vcur = Vnext; Vnext = x;
     }
     ++sweep;
-    cudaMemsetAsync(norms_dev, 0, 2 * sizeof(double), st);
-    k_offnorm<C><<<64, 256, 0, st>>>(Acur, n, norms_dev); count_launch();
-    cudaError_t e = cudaMemcpyAsync(h, norms_dev, 2 * sizeof(double), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return -1;
+    if (off_norm()) return -1;
     // converged below tol * ||A||_F, or stalled at the rounding floor (no halving in a sweep)
     const double off = sqrt(h[0]), nrm = sqrt(h[0] + h[1]);
     const double floor_rel = sizeof(C) == 16 ? 1e-10 : 1e-4;
@@ -530,13 +544,13 @@ __global__ void k_sort_eig(const double2* A, const double2* V, int n, double* ei
 }
 
 int la_jacobi_eigh(double2* A, int n, double2* U, double* eig, double2* ws, double* norms_dev,
-                   cudaStream_t st, int max_sweeps, double tol, int* sweeps_out) {
+                   cudaStream_t st, int max_sweeps, double tol, bool check_first, int* sweeps_out) {
   // ws: 3 n*n + n + 2 complex (V, then the A copy, V copy and rotations of a round)
   double2* V = ws;
   bool conv = false;
   double2 *Af = nullptr, *Vf = nullptr;
-  const int sweep = jacobi_sweeps<double2>(A, n, V, ws + (int64_t)n * n, norms_dev, st, max_sweeps, tol, &conv, &Af,
-                                           &Vf);
+  const int sweep = jacobi_sweeps<double2>(A, n, V, ws + (int64_t)n * n, norms_dev, st, max_sweeps, tol, check_first,
+                                           &conv, &Af, &Vf);
   if (sweep < 0) return cuda_status(cudaGetLastError(), "jacobi");
   if (sweeps_out) *sweeps_out = sweep;
   k_sort_eig<<<n, 128, 0, st>>>(Af, Vf, n, eig, U); count_launch();
@@ -552,7 +566,8 @@ int la_jacobi_rotate32(float2* A, int n, float2* V, float2* ws, double* norms_de
                        double tol, int* sweeps_out) {
   bool conv = false;
   float2 *Af = nullptr, *Vf = nullptr;
-  const int sweep = jacobi_sweeps<float2>(A, n, V, ws, norms_dev, st, max_sweeps, tol, &conv, &Af, &Vf);
+  const int sweep = jacobi_sweeps<float2>(A, n, V, ws, norms_dev, st, max_sweeps, tol, false, &conv, &Af,
+                                          &Vf);
   if (sweep < 0) return cuda_status(cudaGetLastError(), "jacobi (FP32)");
   if (Vf != V) {
     cudaError_t e = cudaMemcpyAsync(V, Vf, sizeof(float2) * (size_t)n * n, cudaMemcpyDeviceToDevice, st);
@@ -560,6 +575,34 @@ int la_jacobi_rotate32(float2* A, int n, float2* V, float2* ws, double* norms_de
   }
   if (sweeps_out) *sweeps_out = sweep;
   return PW_OK;
+}
+
+// I + K, K anti-Hermitian, K_ij the tangent of the Jacobi rotation of the pair (i, j) of a nearly
+// diagonal Hermitian A (A_ij / (A_jj - A_ii) to first order): for well separated levels I + K is
+// the first-order correction of the eigenvectors, and for a close pair alone its columns, made
+// orthonormal, are the rotation itself
+__global__ void k_eig_correction(const double2* __restrict__ A, int n, double2* __restrict__ K) {
+  const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (idx >= (int64_t)n * n) return;
+  const int i = (int)(idx % n), j = (int)(idx / n);
+  if (i == j) {
+    K[idx] = make_double2(1.0, 0.0);
+    return;
+  }
+  const int p = min(i, j), q = max(i, j);
+  const double2 b = A[p + (int64_t)q * n];
+  const double ab = hypot(b.x, b.y);
+  double2 k = make_double2(0.0, 0.0);
+  if (ab > 1e-300) {
+    const double tau = (A[q + (int64_t)q * n].x - A[p + (int64_t)p * n].x) / (2.0 * ab);
+    const double t = (tau >= 0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau)) / ab;
+    k = i < j ? make_double2(t * b.x, t * b.y) : make_double2(-t * b.x, t * b.y);
+  }
+  K[idx] = k;
+}
+cudaError_t la_eig_correction(const double2* A, int n, double2* K, cudaStream_t st) {
+  k_eig_correction<<<(unsigned)(((int64_t)n * n + 255) / 256), 256, 0, st>>>(A, n, K); count_launch();
+  return cudaGetLastError();
 }
 
 // ---- column reductions ------------------------------------------------------------

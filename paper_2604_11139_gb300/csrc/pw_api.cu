@@ -901,15 +901,20 @@ int check_flag(pw_ctx* ctx, int* flag_dev, const char* what) {
 }
 
 // Hermitian eigensolve of a reduced matrix A (n x n, lda n, destroyed): U (n x n) and eig
-// (device, ascending); jac: 3 n*n + n + 2 complex128, norms: 2 doubles (device).  From n = 128 an
+// (device, ascending); jac: 3 n*n + n + 2 complex128, norms: 2 doubles (device).  From n = 16 an
 // FP32 Jacobi pre-rotation first: V32 brings A near diagonal at the FP32 rate; V = V32 made
-// unitary in FP64 (Cholesky-QR), A' = V^dagger A V by FP64-accurate GEMMs is then a similarity
-// transform of A to rounding and nearly diagonal, so the FP64 Jacobi on A' needs only a few
-// sweeps; U = V U'.
-constexpr int kMixedEigMin = 128;
+// unitary in FP64 (Cholesky-QR), A' = V^dagger A V is then a similarity transform of A to rounding
+// and nearly diagonal.  Two corrections V <- V (I + K), each followed by Cholesky-QR, square the
+// remaining off-diagonal part (K_ij is the tangent of the pair's Jacobi rotation, A'_ij / (A'_jj -
+// A'_ii) to first order).  The FP64 Jacobi finishes on A' (no sweep when nothing is left), U = V U'.
+// A sweep of FP64 rounds takes 10 ms at n = 512 (two launches a round, a chain of square roots and
+// divisions), a correction 2 ms; without the corrections two sweeps were needed there, and below
+// n = 128, without FP32 rotations, seven or eight (5 ms each at n = 96).
+constexpr int kMixedEigMin = 16;
+constexpr int kEigCorrections = 2;
 int eigh_impl(pw_ctx* ctx, double2* A, int n, double2* U, double* eig, double2* jac, double* norms, int* sweeps) {
   const cudaStream_t st = ctx->stream;
-  if (n < kMixedEigMin) return la_jacobi_eigh(A, n, U, eig, jac, norms, st, 40, 1e-13, sweeps);
+  if (n < kMixedEigMin) return la_jacobi_eigh(A, n, U, eig, jac, norms, st, 40, 1e-13, false, sweeps);
   const size_t nn = (size_t)n * n;
   const size_t bytes = sizeof(double2) * 5 * nn + sizeof(float2) * (4 * nn + n + 2) + 64;
   WS(mixb, unsigned char, WS_EIGMIX, bytes);
@@ -922,29 +927,35 @@ int eigh_impl(pw_ctx* ctx, double2* A, int n, double2* U, double* eig, double2* 
   float2* V32 = A32 + nn;
   float2* w32 = V32 + nn;
   int* flag = (int*)(w32 + 2 * nn + n + 2);
+  // products of n x n matrices: tiles of 16 on the FP64 pipe beat slicing and digits up to 160
+  auto mul = [&](int ta, int tb, const double2* X, const double2* Y, double2* out, int tri, const char* what) -> int {
+    if (n > 160) return cg<double>(ctx, ta, tb, n, n, n, X, n, Y, n, epi<double>(EPI_STORE, out, n), 1, nullptr, st, tri, what);
+    CU_TRY(launch_cgemm<double>(ta, tb, n, n, n, X, n, Y, n, epi<double>(EPI_STORE, out, n), 1, nullptr, st, tri), what);
+    return PW_OK;
+  };
   CU_TRY(cudaMemsetAsync(flag, 0, sizeof(int), st), "flag reset");
   CU_TRY(la_to_c64(A, n, A32, n, n, n, st), "eig: to c64");
   int sw32 = 0, sw64 = 0;
   PW_TRY(la_jacobi_rotate32(A32, n, V32, w32, norms, st, 30, 1e-6, &sw32));
   CU_TRY(la_to_c128(V32, n, V, n, n, n, st), "eig: to c128");
-  // Vo = V L^{-dagger}, L L^dagger = V^dagger V
-  PW_TRY(cg<double>(ctx, 1, 0, n, n, n, V, n, V, n, epi<double>(EPI_STORE, Gv, n), 1, nullptr, st, GEMM_FULL,
-                    "eig basis Gram"));
-  CU_TRY(la_herm_sym(Gv, n, n, st), "eig basis Gram sym");
-  CU_TRY(la_cholesky(Gv, n, n, flag, st), "eig basis Cholesky");
-  CU_TRY(la_trinv_lower(Gv, n, n, Lv, n, T, st), "eig basis triangular inverse");
-  PW_TRY(cg<double>(ctx, 0, 1, n, n, n, V, n, Lv, n, epi<double>(EPI_STORE, Vo, n), 1, nullptr, st, GEMM_B_UPPER,
-                    "eig basis orthonormalisation"));
+  for (int it = 0;; ++it) {
+    // Vo = V L^{-dagger}, L L^dagger = V^dagger V
+    PW_TRY(mul(1, 0, V, V, Gv, GEMM_FULL, "eig basis Gram"));
+    CU_TRY(la_herm_sym(Gv, n, n, st), "eig basis Gram sym");
+    CU_TRY(la_cholesky(Gv, n, n, flag, st), "eig basis Cholesky");
+    CU_TRY(la_trinv_lower(Gv, n, n, Lv, n, T, st), "eig basis triangular inverse");
+    PW_TRY(mul(0, 1, V, Lv, Vo, GEMM_B_UPPER, "eig basis orthonormalisation"));
+    // A' = Vo^dagger A Vo
+    PW_TRY(mul(0, 0, A, Vo, T, GEMM_FULL, "eig rotate 1"));
+    PW_TRY(mul(1, 0, Vo, T, Gv, GEMM_FULL, "eig rotate 2"));
+    CU_TRY(la_herm_sym(Gv, n, n, st), "eig rotated sym");
+    if (it == kEigCorrections) break;
+    CU_TRY(la_eig_correction(Gv, n, T, st), "eig correction");
+    PW_TRY(mul(0, 0, Vo, T, V, GEMM_FULL, "eig corrected basis"));
+  }
   PW_TRY(check_flag(ctx, flag, "eigensolver basis Cholesky"));
-  // A' = Vo^dagger A Vo (into A), FP64 Jacobi on it, U = Vo U'
-  PW_TRY(cg<double>(ctx, 0, 0, n, n, n, A, n, Vo, n, epi<double>(EPI_STORE, T, n), 1, nullptr, st, GEMM_FULL,
-                    "eig rotate 1"));
-  PW_TRY(cg<double>(ctx, 1, 0, n, n, n, Vo, n, T, n, epi<double>(EPI_STORE, A, n), 1, nullptr, st, GEMM_FULL,
-                    "eig rotate 2"));
-  CU_TRY(la_herm_sym(A, n, n, st), "eig rotated sym");
-  PW_TRY(la_jacobi_eigh(A, n, T, eig, jac, norms, st, 40, 1e-13, &sw64));
-  PW_TRY(cg<double>(ctx, 0, 0, n, n, n, Vo, n, T, n, epi<double>(EPI_STORE, U, n), 1, nullptr, st, GEMM_FULL,
-                    "eig back-rotation"));
+  PW_TRY(la_jacobi_eigh(Gv, n, T, eig, jac, norms, st, 40, 1e-13, true, &sw64));
+  PW_TRY(mul(0, 0, Vo, T, U, GEMM_FULL, "eig back-rotation"));
   if (sweeps) *sweeps = sw64;
   return PW_OK;
 }
