@@ -290,8 +290,8 @@ int forward_t(pw_diff* df, double2* psi, int64_t ld, int steps, const double2* v
     PW_TRY(api::rr(ctx, psi, ld, M, df->eig_h.data(), df->Qt[t], df->Xt[t], df->lamt[t]));
     // R^H = Y_m^H Q (lower triangular), kept as its inverse
     const int ns = api::gemm_nsplit(M, M, N);
-    CU_TRY(launch_cgemm<double>(1, 0, M, M, N, df->Y64, N, df->Qt[t], N, epi64(EPI_STORE, df->mT, M), ns, df->gsplit,
-                                st), "R^H");
+    PW_TRY(api::gemm64(ctx, 1, 0, M, M, N, df->Y64, N, df->Qt[t], N, epi64(EPI_STORE, df->mT, M), ns, df->gsplit,
+           "R^H"));
     CU_TRY(la_zero_upper(df->mT, M, M, st), "R^H lower");
     CU_TRY(la_trinv_lower(df->mT, M, M, df->Lt[t], M, df->mG, st), "R^H inverse");
     a = df->eig_h[M - 1];
@@ -336,8 +336,8 @@ int contract(pw_diff* df, const cplx<T>* a, const cplx<T>* b, const cplx<T>* Ca,
       ca64 = df->cz64;
       cb64 = df->ck64;
     }
-    CU_TRY(launch_cgemm<double>(0, 1, np, np, M, ca64, np, cb64, np, epi64(EPI_ACCUM, df->dDacc, np, weight), 1,
-                                nullptr, st), "adjoint D contraction");
+    PW_TRY(api::gemm64(ctx, 0, 1, np, np, M, ca64, np, cb64, np, epi64(EPI_ACCUM, df->dDacc, np, weight), 1,
+                                nullptr, "adjoint D contraction"));
   }
   return PW_OK;
 }
@@ -366,44 +366,36 @@ int backward_t(pw_diff* df, const double* eigbar, const double2* psibar, int64_t
     const bool last = (t == df->cycles - 1);
     const double2 *Q = df->Qt[t], *X = df->Xt[t];
     // Qb = Psib X^H
-    CU_TRY(launch_cgemm<double>(0, 1, N, M, M, df->PB, N, X, M, epi64(EPI_STORE, df->QB, N), 1, nullptr, st),
-           "Qb = Psib X^H");
+    PW_TRY(api::gemm64(ctx, 0, 1, N, M, M, df->PB, N, X, M, epi64(EPI_STORE, df->QB, N), 1, nullptr, "Qb = Psib X^H"));
     const bool keep_any = split < 0 || (split > 0 && split < M);
     if (last && (have_lb || keep_any)) {
       // K = X^H (Q^H Psib); G; Ab = Herm(X G X^H)
-      CU_TRY(launch_cgemm<double>(1, 0, M, M, N, Q, N, df->PB, N, epi64(EPI_STORE, df->mT, M), ns, df->gsplit, st),
-             "Q^H Psib");
-      CU_TRY(launch_cgemm<double>(1, 0, M, M, M, X, M, df->mT, M, epi64(EPI_STORE, df->mK, M), 1, nullptr, st),
-             "K");
+      PW_TRY(api::gemm64(ctx, 1, 0, M, M, N, Q, N, df->PB, N, epi64(EPI_STORE, df->mT, M), ns, df->gsplit, "Q^H Psib"));
+      PW_TRY(api::gemm64(ctx, 1, 0, M, M, M, X, M, df->mT, M, epi64(EPI_STORE, df->mK, M), 1, nullptr, "K"));
       k_eig_adjoint<<<g2, b2, 0, st>>>(df->mK, df->lamt[t], have_lb ? df->lamb : nullptr, M, split, df->mG);
       count_launch();
-      CU_TRY(launch_cgemm<double>(0, 1, M, M, M, df->mG, M, X, M, epi64(EPI_STORE, df->mT, M), 1, nullptr, st),
-             "G X^H");
-      CU_TRY(launch_cgemm<double>(0, 0, M, M, M, X, M, df->mT, M, epi64(EPI_STORE, df->mA, M), 1, nullptr, st),
-             "X G X^H");
+      PW_TRY(api::gemm64(ctx, 0, 1, M, M, M, df->mG, M, X, M, epi64(EPI_STORE, df->mT, M), 1, nullptr, "G X^H"));
+      PW_TRY(api::gemm64(ctx, 0, 0, M, M, M, X, M, df->mT, M, epi64(EPI_STORE, df->mA, M), 1, nullptr, "X G X^H"));
       CU_TRY(la_herm_sym(df->mA, M, M, st), "Ab Hermitian part");
       // Qb += 2 H Q Ab ; direct parameter terms of A = Q^H H Q
       PW_TRY(api::apply64(ctx, Q, N, M, df->HQ, N));
-      CU_TRY(launch_cgemm<double>(0, 0, N, M, M, df->HQ, N, df->mA, M, epi64(EPI_ACCUM, df->QB, N, 2.0), 1, nullptr,
-                                  st), "Qb += 2 HQ Ab");
-      CU_TRY(launch_cgemm<double>(0, 0, N, M, M, Q, N, df->mA, M, epi64(EPI_STORE, df->QA, N), 1, nullptr, st),
-             "Q Ab");
+      PW_TRY(api::gemm64(ctx, 0, 0, N, M, M, df->HQ, N, df->mA, M, epi64(EPI_ACCUM, df->QB, N, 2.0), 1, nullptr,
+             "Qb += 2 HQ Ab"));
+      PW_TRY(api::gemm64(ctx, 0, 0, N, M, M, Q, N, df->mA, M, epi64(EPI_STORE, df->QA, N), 1, nullptr, "Q Ab"));
       if (np > 0) {
         const int nsp = api::gemm_nsplit(np, M, N);
-        CU_TRY(launch_cgemm<double>(1, 0, np, M, N, ctx->P64, N, df->QA, N, epi64(EPI_STORE, df->CA, np), nsp,
-                                    df->gsplit, st), "P^H Q Ab");
-        CU_TRY(launch_cgemm<double>(1, 0, np, M, N, ctx->P64, N, Q, N, epi64(EPI_STORE, df->CQ, np), nsp,
-                                    df->gsplit, st), "P^H Q");
+        PW_TRY(api::gemm64(ctx, 1, 0, np, M, N, ctx->P64, N, df->QA, N, epi64(EPI_STORE, df->CA, np), nsp,
+                                    df->gsplit, "P^H Q Ab"));
+        PW_TRY(api::gemm64(ctx, 1, 0, np, M, N, ctx->P64, N, Q, N, epi64(EPI_STORE, df->CQ, np), nsp,
+                                    df->gsplit, "P^H Q"));
       }
       PW_TRY(contract<double>(df, df->QA, Q, df->CA, df->CQ, 1.0));
     }
     // span projection and R^-H:  Ym_b = (Qb - Q (Q^H Qb)) (R^H)^-1
-    CU_TRY(launch_cgemm<double>(1, 0, M, M, N, Q, N, df->QB, N, epi64(EPI_STORE, df->mT, M), ns, df->gsplit, st),
-           "Q^H Qb");
-    CU_TRY(launch_cgemm<double>(0, 0, N, M, M, Q, N, df->mT, M, epi64(EPI_ACCUM, df->QB, N, -1.0), 1, nullptr, st),
-           "project out span");
-    CU_TRY(launch_cgemm<double>(0, 0, N, M, M, df->QB, N, df->Lt[t], M, epi64(EPI_STORE, df->HQ, N), 1, nullptr, st),
-           "Ym_b");
+    PW_TRY(api::gemm64(ctx, 1, 0, M, M, N, Q, N, df->QB, N, epi64(EPI_STORE, df->mT, M), ns, df->gsplit, "Q^H Qb"));
+    PW_TRY(api::gemm64(ctx, 0, 0, N, M, M, Q, N, df->mT, M, epi64(EPI_ACCUM, df->QB, N, -1.0), 1, nullptr,
+           "project out span"));
+    PW_TRY(api::gemm64(ctx, 0, 0, N, M, M, df->QB, N, df->Lt[t], M, epi64(EPI_STORE, df->HQ, N), 1, nullptr, "Ym_b"));
     // adjoint recurrence, from Z_m down to Z_0
     C* zbuf[3] = {(C*)df->zb[0], (C*)df->zb[1], (C*)df->zb[2]};
     auto zl = [&](int k) { return zbuf[k % 3]; };

@@ -18,6 +18,9 @@ int rr(pw_ctx* ctx, double2* Y, int64_t ldy, int m, double* eig_h, double2* q_ou
 // largest Rayleigh quotient of psi (nband > 0) and the Lanczos upper bound (steps > 0)
 int bounds(pw_ctx* ctx, const double2* psi, int64_t ld, int nband, int steps, const double2* v0, double* rq_max,
            double* upper);
+// launch_cgemm<double> (without structure), on the tensor cores with eight digits where it is large
+int gemm64(pw_ctx* ctx, int ta, int tb, int M, int N, int K, const double2* A, int64_t lda, const double2* B,
+           int64_t ldb, const Epi<double>& e, int nsplit, double2* ws, const char* where);
 int fft_band_batch(const pw_ctx* ctx, int nband, size_t elem);
 int gemm_nsplit(int m, int n, int k);
 }  // namespace api

@@ -403,7 +403,8 @@ int ensure_ozp(pw_ctx* ctx) {
 // columns (matrix-vector forms, memory-bound); op(A) = P^dagger or P uses the context's cached
 // digit planes.  dfma_ns / dfma_ws: split-K of the DFMA form.
 int zgemm(pw_ctx* ctx, int ta, int tb, int M, int N, int K, const double2* A, int64_t lda, const double2* B,
-          int64_t ldb, const Epi<double>& e, int dfma_ns, double2* dfma_ws, int tri, const char* where) {
+          int64_t ldb, const Epi<double>& e, int dfma_ns, double2* dfma_ws, int tri, const char* where,
+          int digits = oz::kDigits) {
   if (M <= 0 || N <= 0) return PW_OK;
   const cudaStream_t st = ctx->stream;
   if (!ctx->fp64_tc || N <= 4 || K <= 0 || !oz::available()) {
@@ -412,9 +413,9 @@ int zgemm(pw_ctx* ctx, int ta, int tb, int M, int N, int K, const double2* A, in
   }
   PW_TRY(ensure_err_flag(ctx));
   const int lower = (tri == GEMM_LOWER_OUT);
-  oz::Digits Ad{nullptr, 2 * M, 2 * K, oz::digit_pitch(2 * K), 0, nullptr};
+  oz::Digits Ad{nullptr, 2 * M, 2 * K, oz::digit_pitch(2 * K), 0, nullptr, digits};
   Ad.plane = (int64_t)Ad.rows * Ad.pitch;
-  const bool is_p = (A == ctx->P64 && ctx->nproj > 0 && lda == ctx->npw);
+  const bool is_p = (A == ctx->P64 && ctx->nproj > 0 && lda == ctx->npw && digits == oz::kDigits);
   if (is_p && ta == 1 && M == ctx->nproj && K == ctx->npw) {
     PW_TRY(ensure_ozp(ctx));
     Ad.dig = (const __nv_bfloat16*)ctx->ozPH;
@@ -424,18 +425,20 @@ int zgemm(pw_ctx* ctx, int ta, int tb, int M, int N, int K, const double2* A, in
     Ad.dig = (const __nv_bfloat16*)ctx->ozP;
     Ad.exp = ctx->ozP_exp;
   }
-  oz::Digits Bd{nullptr, N, 2 * K, oz::digit_pitch(2 * K), 0, nullptr};
+  oz::Digits Bd{nullptr, N, 2 * K, oz::digit_pitch(2 * K), 0, nullptr, digits};
   Bd.plane = (int64_t)Bd.rows * Bd.pitch;
   WS(amax, unsigned long long, WS_OZAMAX, std::max(M, N));
   WS(ex, int, WS_OZEXP, (size_t)M + N);
   if (!Ad.dig) {
-    WS(ad, __nv_bfloat16, WS_OZA, (size_t)oz::kDigits * Ad.plane);
-    CU_TRY(oz::slice(A, ta ? lda : 1, ta ? 1 : lda, ta, M, K, 1, ad, Ad.pitch, Ad.plane, amax, ex, st), where);
+    WS(ad, __nv_bfloat16, WS_OZA, (size_t)digits * Ad.plane);
+    CU_TRY(oz::slice(A, ta ? lda : 1, ta ? 1 : lda, ta, M, K, 1, ad, Ad.pitch, Ad.plane, amax, ex, st, digits),
+           where);
     Ad.dig = ad;
     Ad.exp = ex;
   }
-  WS(bd, __nv_bfloat16, WS_OZB, (size_t)oz::kDigits * Bd.plane);
-  CU_TRY(oz::slice(B, tb ? 1 : ldb, tb ? ldb : 1, tb, N, K, 0, bd, Bd.pitch, Bd.plane, amax, ex + M, st), where);
+  WS(bd, __nv_bfloat16, WS_OZB, (size_t)digits * Bd.plane);
+  CU_TRY(oz::slice(B, tb ? 1 : ldb, tb ? ldb : 1, tb, N, K, 0, bd, Bd.pitch, Bd.plane, amax, ex + M, st, digits),
+         where);
   Bd.dig = bd;
   Bd.exp = ex + M;
   const int ns = oz::split_count(2 * M, N, 2 * K, lower);
@@ -927,9 +930,12 @@ int eigh_impl(pw_ctx* ctx, double2* A, int n, double2* U, double* eig, double2* 
   float2* V32 = A32 + nn;
   float2* w32 = V32 + nn;
   int* flag = (int*)(w32 + 2 * nn + n + 2);
-  // products of n x n matrices: tiles of 16 on the FP64 pipe beat slicing and digits up to 160
+  // products of n x n matrices: tiles of 16 on the FP64 pipe beat slicing and digits up to 160;
+  // eight digits, or the rounding of A' alone (1e-13 of its norm at n = 512) costs another sweep
   auto mul = [&](int ta, int tb, const double2* X, const double2* Y, double2* out, int tri, const char* what) -> int {
-    if (n > 160) return cg<double>(ctx, ta, tb, n, n, n, X, n, Y, n, epi<double>(EPI_STORE, out, n), 1, nullptr, st, tri, what);
+    if (n > 160)
+      return zgemm(ctx, ta, tb, n, n, n, X, n, Y, n, epi<double>(EPI_STORE, out, n), 1, nullptr, tri, what,
+                   oz::kDigitsFull);
     CU_TRY(launch_cgemm<double>(ta, tb, n, n, n, X, n, Y, n, epi<double>(EPI_STORE, out, n), 1, nullptr, st, tri), what);
     return PW_OK;
   };
@@ -1604,6 +1610,16 @@ template int recur<double>(pw_ctx*, const double2*, int64_t, const double2*, int
                            double, double, double2*);
 template int recur<float>(pw_ctx*, const float2*, int64_t, const float2*, int64_t, float2*, int64_t, int, double,
                           double, double, float2*);
+// From 2^25 complex products the digits and their products (0.2 ms at 14771 x 128 x 128) beat the
+// FP64 pipe (4 FMAs each: 0.22 ms at 2^25, 1.6 ms at 14771 x 128 x 128).  Eight digits: the result is
+// as close to exact as the FMAs' (a product that the filter and Rayleigh-Ritz take with seven).
+int gemm64(pw_ctx* ctx, int ta, int tb, int M, int N, int K, const double2* A, int64_t lda, const double2* B,
+           int64_t ldb, const Epi<double>& e, int nsplit, double2* ws, const char* where) {
+  if ((double)M * N * K >= (double)(1 << 25))
+    return zgemm(ctx, ta, tb, M, N, K, A, lda, B, ldb, e, nsplit, ws, GEMM_FULL, where, oz::kDigitsFull);
+  CU_TRY(launch_cgemm<double>(ta, tb, M, N, K, A, lda, B, ldb, e, nsplit, ws, ctx->stream), where);
+  return PW_OK;
+}
 int rr(pw_ctx* ctx, double2* Y, int64_t ldy, int m, double* eig_h, double2* q_out, double2* x_out,
        double* eig_dev_out) {
   return rr_impl(ctx, Y, ldy, m, nullptr, eig_h, nullptr, q_out, x_out, eig_dev_out);

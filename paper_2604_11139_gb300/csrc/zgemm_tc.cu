@@ -14,7 +14,9 @@
 // 64-bit integer arithmetic, v = sum_d acc_d 2^(7 (6 - d)) < 2^62.1, and v is added to an FP64
 // running sum; the result is 2^(e_row + e_col - 56) times that sum.  The dropped products
 // (s + t >= 7) are below 2^-44 of |a_max| |b_max| per K element, the FP64 rounding of v and of
-// the running sum are ordinary FP64 roundings.
+// the running sum are ordinary FP64 roundings.  With eight digits (56 bits, 36 products, eight
+// accumulators, v in two 64-bit parts) everything moves by seven bits: the dropped products are
+// below 2^-51.
 //
 // Complex operands are realified: op(A) (M x K) becomes the 2M x 2K real matrix whose rows 2i
 // and 2i+1 are (Re a, -Im a) and (Im a, Re a) per entry, op(B) (K x N) the N x 2K matrix of
@@ -46,23 +48,24 @@ namespace pw {
 namespace oz {
 using namespace tcp;
 
-constexpr int S = kDigits;
 constexpr int BM = 128, BN = 64, BK = 32;
 constexpr int KC = 256;                      // K elements per exact chunk
 constexpr int SLICES_PER_CHUNK = KC / BK;    // 8
 constexpr int STAGES = 2;
 constexpr int A_TILE = BM * BK * 2;          // 8 KB per digit plane
 constexpr int B_TILE = BN * BK * 2;          // 4 KB per digit plane
-constexpr int STAGE_BYTES = S * (A_TILE + B_TILE);
-constexpr int SMEM = STAGES * STAGE_BYTES + 1024 + 256;
+constexpr int stage_bytes(int S) { return S * (A_TILE + B_TILE); }
+constexpr int smem_bytes(int S) { return STAGES * stage_bytes(S) + 1024 + 256; }
 constexpr int EPI_WARPS = 16;                // 4 per TMEM lane quarter, 16 columns each
 constexpr int THREADS = 32 * (2 + EPI_WARPS);
-constexpr uint32_t kTmemCols = 512;          // 7 accumulators x 64 columns = 448 used
+constexpr uint32_t kTmemCols = 512;          // 7 (8) accumulators x 64 columns = 448 (512) used
 constexpr uint32_t kSpin = 1u << 24;
 constexpr uint32_t kSpinTest = 1u << 12;
 
 int64_t digit_pitch(int k2) { return ((int64_t)k2 + 7) / 8 * 8; }
-size_t digit_bytes(int rows, int k2) { return sizeof(__nv_bfloat16) * (size_t)S * rows * digit_pitch(k2); }
+size_t digit_bytes(int rows, int k2, int digits) {
+  return sizeof(__nv_bfloat16) * (size_t)digits * rows * digit_pitch(k2);
+}
 
 // ---------------------------------------------------------------------------------------------
 // slicing
@@ -98,21 +101,25 @@ __global__ void __launch_bounds__(256) k_oz_rowmax(const double2* __restrict__ X
   for (int i = 0; i < 4; ++i) {
     const int rr = ty + 8 * i;
     const double2 v = sm[rr][tx];
-    double m = fmax(fabs(v.x), fabs(v.y));
+    double m = isfinite(v.x) && isfinite(v.y) ? fmax(fabs(v.x), fabs(v.y)) : INFINITY;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (tx == 0 && r0 + rr < R && m > 0.0) atomicMax(&amax[r0 + rr], (unsigned long long)__double_as_longlong(m));
   }
 }
 
-// exponent e with max |entry| 2^-e in [1/4, 1/2): e = ilogb(max) + 2 (0 for a zero row)
+// exponent e with max |entry| 2^-e in [1/4, 1/2): e = ilogb(max) + 2 (0 for a zero row); kNotFinite
+// (all digits then come out 0) for a row with an infinity or NaN
+constexpr int kNotFinite = 1 << 24;
 __device__ __forceinline__ int row_exp(unsigned long long bits) {
   if (bits == 0ull) return 0;
+  if (bits >= 0x7ff0000000000000ull) return kNotFinite;
   return ilogb(__longlong_as_double((long long)bits)) + 2;
 }
 
-// N = round(x 2^(49 - e)) as an integer (|N| <= 2^48 since |x| < 2^(e - 1)), by integer
+// N = round(x 2^(7 S - e)) as an integer (|N| <= 2^(7 S - 1) since |x| < 2^(e - 1)), by integer
 // arithmetic on the FP64 representation (round half away from zero)
+template <int S>
 __device__ __forceinline__ long long scaled_int(double x, int e) {
   const long long bits = __double_as_longlong(x);
   const int bexp = (int)((bits >> 52) & 0x7ff);
@@ -124,7 +131,7 @@ __device__ __forceinline__ long long scaled_int(double x, int e) {
     m |= 0x10000000000000ll;
     E = bexp - 1075;
   }
-  const int sh = E + 49 - e;
+  const int sh = E + 7 * S - e;
   long long n;
   if (m == 0) n = 0;
   else if (sh >= 0) n = m << sh;
@@ -133,8 +140,9 @@ __device__ __forceinline__ long long scaled_int(double x, int e) {
   return bits < 0 ? -n : n;
 }
 
-// balanced base-128 digits of n (|n| <= 2^48): n = sum_s d_s 128^(6 - s); the six lower digits
+// balanced base-128 digits of n (|n| <= 2^(7 S - 1)): n = sum_s d_s 128^(S - 1 - s); the lower digits
 // are taken in [-64, 63] and the leading digit is what remains, which is within [-64, 64]
+template <int S>
 __device__ __forceinline__ void digits7(long long n, float (&d)[S]) {
 #pragma unroll
   for (int s = S - 1; s >= 1; --s) {
@@ -145,6 +153,7 @@ __device__ __forceinline__ void digits7(long long n, float (&d)[S]) {
   d[0] = (float)n;
 }
 
+template <int S>
 __global__ void __launch_bounds__(256) k_oz_slice(const double2* __restrict__ X, int64_t sr, int64_t sl, int cj,
                                                   int R, int K, int aform, __nv_bfloat16* __restrict__ dig,
                                                   int64_t pitch, int64_t plane,
@@ -162,8 +171,8 @@ __global__ void __launch_bounds__(256) k_oz_slice(const double2* __restrict__ X,
     if (blockIdx.y == 0 && tx == 0) ex[r] = e;
     const double2 v = sm[rr][tx];
     float dr[S], di[S];
-    digits7(scaled_int(v.x, e), dr);
-    digits7(scaled_int(v.y, e), di);
+    digits7<S>(scaled_int<S>(v.x, e), dr);
+    digits7<S>(scaled_int<S>(v.y, e), di);
 #pragma unroll
     for (int s = 0; s < S; ++s) {
       __nv_bfloat16* p = dig + (int64_t)s * plane + 2 * (int64_t)l;
@@ -227,8 +236,10 @@ __device__ __forceinline__ void oz_epi(const Epi<double>& e, int R, int j, doubl
   }
 }
 
+template <int S>
 __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ CUtensorMap tmA,
                                                         const __grid_constant__ CUtensorMap tmB, Args a) {
+  constexpr int STAGE_BYTES = stage_bytes(S);
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* full = (uint64_t*)(base + STAGES * STAGE_BYTES);
@@ -361,44 +372,57 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
           break;
         }
         fence_after();
-        // v = sum_d acc_d 128^(6 - d) from 32-bit pairs, |128 acc_d + acc_(d+1)| < 2^30
-        long long v[16];
+        // the chunk's value sum_d acc_d 128^(S - 1 - d) = 2^28 H + L from 32-bit pairs, |128 acc_d +
+        // acc_(d+1)| < 2^31: H from the first S - 4 accumulators, L from the last four
+        [[maybe_unused]] long long hi[16];
+        long long lo[16];
 #pragma unroll
         for (int g = 0; g < 16; g += 8) {
-          uint32_t r[7][8];
-          auto ival = [&](int d, int i) { return __float2int_rn(__uint_as_float(r[d][i])); };
+          constexpr int H = S - 4;
+          uint32_t r[S][8];
+          auto pair = [&](int d, int i) {
+            return __float2int_rn(__uint_as_float(r[d][i])) * 128 + __float2int_rn(__uint_as_float(r[d + 1][i]));
+          };
 #pragma unroll
-          for (int d = 3; d < 7; ++d) tmem_ld8_async(tl + (uint32_t)(d * BN + g), r[d]);
+          for (int d = H; d < S; ++d) tmem_ld8_async(tl + (uint32_t)(d * BN + g), r[d]);
 #pragma unroll
-          for (int d = 3; d < 7; ++d) tmem_wait_ld8(r[d]);
+          for (int d = H; d < S; ++d) tmem_wait_ld8(r[d]);
 #pragma unroll
-          for (int d = 0; d < 3; ++d) tmem_ld8_async(tl + (uint32_t)(d * BN + g), r[d]);
+          for (int d = 0; d < H; ++d) tmem_ld8_async(tl + (uint32_t)(d * BN + g), r[d]);
 #pragma unroll
-          for (int i = 0; i < 8; ++i)
-            v[g + i] = (long long)(ival(3, i) * 128 + ival(4, i)) * (1 << 14) + (ival(5, i) * 128 + ival(6, i));
+          for (int i = 0; i < 8; ++i) lo[g + i] = (long long)pair(H, i) * (1 << 14) + pair(H + 2, i);
 #pragma unroll
-          for (int d = 0; d < 3; ++d) tmem_wait_ld8(r[d]);
+          for (int d = 0; d < H; ++d) tmem_wait_ld8(r[d]);
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
-            v[g + i] += (long long)(ival(1, i) * 128 + ival(2, i)) * (1 << 28);
-            v[g + i] += (long long)(ival(0, i) * 1024) << 32;
+            if constexpr (S == 7) {  // 2^28 H + L < 2^62.1 fits 64 bits
+              lo[g + i] += (long long)pair(1, i) * (1 << 28);
+              lo[g + i] += (long long)(__float2int_rn(__uint_as_float(r[0][i])) * 1024) << 32;
+            } else {
+              hi[g + i] = (long long)pair(0, i) * (1 << 14) + pair(2, i);
+            }
           }
         }
         fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(tempty);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) sum[i] += __ll2double_rn(v[i]);
+        for (int i = 0; i < 16; ++i) {
+          if constexpr (S == 7) sum[i] += __ll2double_rn(lo[i]);
+          else sum[i] += fma(__ll2double_rn(hi[i]), 268435456.0, __ll2double_rn(lo[i]));
+        }
       }
       if (!ok) break;
       const int R = tm * BM + q * 32 + lane;
       if (R < a.M2) {
-        const int er = a.ea[R >> 1] - 56;
+        const int ea = a.ea[R >> 1], er = ea - 7 * (S + 1);
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
           const int j = tn * BN + h * 16 + i;
           if (j < a.N) {
-            const double val = ldexp(sum[i], er + a.eb[j]);
+            const int eb = a.eb[j];
+            const double val = ea == kNotFinite || eb == kNotFinite ? __longlong_as_double(0x7ff8000000000000ll)
+                                                                    : ldexp(sum[i], er + eb);
             if (a.nsplit > 1) a.part[((int64_t)z * a.N + j) * a.M2 + R] = val;
             else oz_epi(a.epi, R, j, val);
           }
@@ -447,14 +471,14 @@ static EncodeFn encode_fn() {
 
 bool available() { return encode_fn() != nullptr; }
 
-// 3-D map over the digit planes [S][rows][pitch], box 32 (K) x box_rows x S, 64-byte swizzle,
+// 3-D map over the digit planes [digits][rows][pitch], box 32 (K) x box_rows x digits, 64-byte swizzle,
 // zero fill beyond k2 and beyond the rows
 static bool make_map(CUtensorMap* m, const Digits& d, int box_rows) {
   EncodeFn fn = encode_fn();
   if (!fn) return false;
-  cuuint64_t dims[3] = {(cuuint64_t)d.k2, (cuuint64_t)d.rows, (cuuint64_t)S};
+  cuuint64_t dims[3] = {(cuuint64_t)d.k2, (cuuint64_t)d.rows, (cuuint64_t)d.digits};
   cuuint64_t strides[2] = {(cuuint64_t)(d.pitch * 2), (cuuint64_t)(d.plane * 2)};
-  cuuint32_t box[3] = {BK, (cuuint32_t)box_rows, S};
+  cuuint32_t box[3] = {BK, (cuuint32_t)box_rows, (cuuint32_t)d.digits};
   cuuint32_t es[3] = {1, 1, 1};
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, (void*)d.dig, dims, strides, box, es,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -462,13 +486,15 @@ static bool make_map(CUtensorMap* m, const Digits& d, int box_rows) {
 }
 
 cudaError_t slice(const double2* X, int64_t sr, int64_t sl, int cj, int R, int K, int aform, __nv_bfloat16* dig,
-                  int64_t pitch, int64_t plane, unsigned long long* amax, int* exp, cudaStream_t st) {
+                  int64_t pitch, int64_t plane, unsigned long long* amax, int* exp, cudaStream_t st, int digits) {
   if (R <= 0 || K <= 0) return cudaSuccess;
   cudaError_t e = cudaMemsetAsync(amax, 0, sizeof(unsigned long long) * (size_t)R, st);
   if (e != cudaSuccess) return e;
   const dim3 grid((R + 31) / 32, (K + 31) / 32);
   k_oz_rowmax<<<grid, 256, 0, st>>>(X, sr, sl, cj, R, K, amax); count_launch();
-  k_oz_slice<<<grid, 256, 0, st>>>(X, sr, sl, cj, R, K, aform, dig, pitch, plane, amax, exp); count_launch();
+  if (digits == kDigits) k_oz_slice<kDigits><<<grid, 256, 0, st>>>(X, sr, sl, cj, R, K, aform, dig, pitch, plane, amax, exp);
+  else k_oz_slice<kDigitsFull><<<grid, 256, 0, st>>>(X, sr, sl, cj, R, K, aform, dig, pitch, plane, amax, exp);
+  count_launch();
   return cudaGetLastError();
 }
 
@@ -520,9 +546,15 @@ cudaError_t gemm(const Digits& A, const Digits& B, int M, int N, int K, const Ep
   int nsm = 148, dev = 0;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const int grid = std::min(a.nunits, nsm);
-  cudaError_t e = cudaFuncSetAttribute(k_oz_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+  const bool full = A.digits == kDigitsFull;
+  if (A.digits != B.digits || (!full && A.digits != kDigits)) return cudaErrorInvalidValue;
+  const void* fn = full ? (const void*)k_oz_gemm<kDigitsFull> : (const void*)k_oz_gemm<kDigits>;
+  const int sm = smem_bytes(A.digits);
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   if (e != cudaSuccess) return e;
-  k_oz_gemm<<<grid, THREADS, SMEM, st>>>(ma, mb, a); count_launch();
+  if (full) k_oz_gemm<kDigitsFull><<<grid, THREADS, sm, st>>>(ma, mb, a);
+  else k_oz_gemm<kDigits><<<grid, THREADS, sm, st>>>(ma, mb, a);
+  count_launch();
   if (nsplit > 1) {
     const int64_t t = (int64_t)a.M2 * N;
     k_oz_reduce<<<(unsigned)((t + 255) / 256), 256, 0, st>>>(a.M2, N, nsplit, part, epi, lower); count_launch();
