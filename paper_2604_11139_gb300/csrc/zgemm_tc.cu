@@ -90,22 +90,43 @@ __device__ __forceinline__ void load_tile(const double2* __restrict__ X, int64_t
   }
 }
 
-__global__ void __launch_bounds__(256) k_oz_rowmax(const double2* __restrict__ X, int64_t sr, int64_t sl, int cj,
-                                                   int R, int K, unsigned long long* __restrict__ amax) {
-  __shared__ double2 sm[32][33];
-  const int r0 = blockIdx.x * 32, l0 = blockIdx.y * 32;
-  load_tile(X, sr, sl, cj, R, K, r0, l0, sm);
+// Largest |Re|, |Im| of every row, as the bits of the FP64 value: integer maxima, since an FP64
+// comparison issues at 2 lanes per clock and SM (three per entry took 0.32 ms where reading the
+// 0.8 GB of 97233 x 512 takes 0.12).  An infinity or NaN gives bits from 0x7ff0... on.
+__device__ __forceinline__ unsigned long long mag_max(unsigned long long m, double2 v) {
+  const unsigned long long x = (unsigned long long)__double_as_longlong(v.x) & 0x7fffffffffffffffull;
+  const unsigned long long y = (unsigned long long)__double_as_longlong(v.y) & 0x7fffffffffffffffull;
+  return max(m, max(x, y));
+}
+// K contiguous: a CTA per row and part of K
+__global__ void __launch_bounds__(256) k_oz_rowmax_k(const double2* __restrict__ X, int64_t sr, int K, int kper,
+                                                     unsigned long long* __restrict__ amax) {
+  __shared__ unsigned long long red[8];
+  const double2* x = X + (int64_t)blockIdx.x * sr;
+  const int l1 = min(K, (int)(blockIdx.y + 1) * kper);
+  unsigned long long m = 0;
+#pragma unroll 4
+  for (int l = blockIdx.y * kper + threadIdx.x; l < l1; l += 256) m = mag_max(m, x[l]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int rr = ty + 8 * i;
-    const double2 v = sm[rr][tx];
-    double m = isfinite(v.x) && isfinite(v.y) ? fmax(fabs(v.x), fabs(v.y)) : INFINITY;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (tx == 0 && r0 + rr < R && m > 0.0) atomicMax(&amax[r0 + rr], (unsigned long long)__double_as_longlong(m));
+  if (threadIdx.x == 0) {
+    for (int i = 1; i < 8; ++i) m = max(m, red[i]);
+    if (m) atomicMax(&amax[blockIdx.x], m);
   }
+}
+// rows contiguous: a thread per row, a part of K per blockIdx.y
+__global__ void __launch_bounds__(256) k_oz_rowmax_r(const double2* __restrict__ X, int64_t sr, int64_t sl, int R,
+                                                     int K, int kper, unsigned long long* __restrict__ amax) {
+  const int r = blockIdx.x * 256 + threadIdx.x;
+  if (r >= R) return;
+  const double2* x = X + (int64_t)r * sr;
+  const int l1 = min(K, (int)(blockIdx.y + 1) * kper);
+  unsigned long long m = 0;
+#pragma unroll 4
+  for (int l = blockIdx.y * kper; l < l1; ++l) m = mag_max(m, x[(int64_t)l * sl]);
+  if (m) atomicMax(&amax[r], m);
 }
 
 // exponent e with max |entry| 2^-e in [1/4, 1/2): e = ilogb(max) + 2 (0 for a zero row); kNotFinite
@@ -147,10 +168,10 @@ __device__ __forceinline__ void digits7(long long n, float (&d)[S]) {
 #pragma unroll
   for (int s = S - 1; s >= 1; --s) {
     const long long q = (n + 64) >> 7;  // floor((n + 64) / 128)
-    d[s] = (float)(n - q * 128);
+    d[s] = (float)(int)(n - q * 128);  // a 32-bit conversion; 64-bit ones run on the FP64 pipe
     n = q;
   }
-  d[0] = (float)n;
+  d[0] = (float)(int)n;
 }
 
 template <int S>
@@ -491,7 +512,16 @@ cudaError_t slice(const double2* X, int64_t sr, int64_t sl, int cj, int R, int K
   cudaError_t e = cudaMemsetAsync(amax, 0, sizeof(unsigned long long) * (size_t)R, st);
   if (e != cudaSuccess) return e;
   const dim3 grid((R + 31) / 32, (K + 31) / 32);
-  k_oz_rowmax<<<grid, 256, 0, st>>>(X, sr, sl, cj, R, K, amax); count_launch();
+  // about 1200 CTAs (8 per SM), none with less than 256 (16 per thread) entries of K
+  if (sl == 1) {
+    const int parts = std::max(1, std::min((1216 + R - 1) / R, K / 256));
+    const int kper = (K + parts - 1) / parts;
+    k_oz_rowmax_k<<<dim3(R, (K + kper - 1) / kper), 256, 0, st>>>(X, sr, K, kper, amax); count_launch();
+  } else {
+    const int rb = (R + 255) / 256, parts = std::max(1, std::min((1216 + rb - 1) / rb, K / 16));
+    const int kper = (K + parts - 1) / parts;
+    k_oz_rowmax_r<<<dim3(rb, (K + kper - 1) / kper), 256, 0, st>>>(X, sr, sl, R, K, kper, amax); count_launch();
+  }
   if (digits == kDigits) k_oz_slice<kDigits><<<grid, 256, 0, st>>>(X, sr, sl, cj, R, K, aform, dig, pitch, plane, amax, exp);
   else k_oz_slice<kDigitsFull><<<grid, 256, 0, st>>>(X, sr, sl, cj, R, K, aform, dig, pitch, plane, amax, exp);
   count_launch();
