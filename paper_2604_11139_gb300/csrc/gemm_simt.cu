@@ -4,6 +4,8 @@
 // products.  On GB300 FP64 has no fast tensor path, so the FP64 forms are
 // DFMA-bound; the kernel keeps a 64x64 complex tile per CTA with a 4x4 register
 // tile per thread and stages 16-deep K slices through shared memory.
+#include <algorithm>
+
 #include "pw_internal.cuh"
 
 namespace pw {
@@ -124,15 +126,18 @@ __global__ void __launch_bounds__(256) k_cgemm(int M, int N, int K, const cplx<T
 // 1024 of 16; complex64 at 64 x 37 x 64 13 and 3.5 us.  Same order of the sum over K as the large tiles without split.
 template <typename T, int TA, int TB>
 __global__ void __launch_bounds__(256) k_cgemm16(int M, int N, int K, const cplx<T>* __restrict__ A, int64_t lda,
-                                                 const cplx<T>* __restrict__ B, int64_t ldb, Epi<T> epi, int tri) {
+                                                 const cplx<T>* __restrict__ B, int64_t ldb, Epi<T> epi, int kchunk,
+                                                 cplx<T>* __restrict__ ws, int tri) {
   using C = cplx<T>;
   __shared__ C As[16][17], Bs[16][17];
   const int x = threadIdx.x & 15, y = threadIdx.x >> 4;
   const int m0 = blockIdx.x * 16, n0 = blockIdx.y * 16;
   if (tri == GEMM_LOWER_OUT && m0 / BM < n0 / BN) return;  // tile above the diagonal
-  const int ke = tri == GEMM_B_UPPER ? min(K, n0 + 16) : K;  // op(B)[k][n] = 0 for k > n
+  const int kb = blockIdx.z * kchunk;
+  int ke = min(K, kb + kchunk);
+  if (tri == GEMM_B_UPPER) ke = min(ke, n0 + 16);  // op(B)[k][n] = 0 for k > n
   C acc = czero<C>();
-  for (int k0 = 0; k0 < ke; k0 += 16) {
+  for (int k0 = kb; k0 < ke; k0 += 16) {
     {
       const int gm = m0 + (TA ? y : x), gk = k0 + (TA ? x : y);
       C v = czero<C>();
@@ -157,7 +162,9 @@ __global__ void __launch_bounds__(256) k_cgemm16(int M, int N, int K, const cplx
     __syncthreads();
   }
   const int m = m0 + x, n = n0 + y;
-  if (m < M && n < N) epi_apply<T>(epi, m, n, acc);
+  if (m >= M || n >= N) return;
+  if (gridDim.z > 1) ws[blockIdx.z * ((int64_t)M * N) + m + (int64_t)n * M] = acc;
+  else epi_apply<T>(epi, m, n, acc);
 }
 
 template <typename T>
@@ -264,6 +271,26 @@ static void launch_gemv(int ta, int M, int K, const cplx<T>* A, int64_t lda, con
 }
 
 template <typename T>
+cudaError_t launch_cgemm16(int ta, int tb, int M, int N, int K, const cplx<T>* A, int64_t lda, const cplx<T>* B,
+                           int64_t ldb, const Epi<T>& epi, int nsplit, cplx<T>* ws, cudaStream_t st, int tri) {
+  if (M <= 0 || N <= 0) return cudaSuccess;
+  int kchunk = (K + std::max(nsplit, 1) - 1) / std::max(nsplit, 1);
+  kchunk = std::max(16, (kchunk + 15) / 16 * 16);
+  nsplit = std::max(1, (K + kchunk - 1) / kchunk);
+  const dim3 g((M + 15) / 16, (N + 15) / 16, nsplit);
+  if (ta == 0 && tb == 0) k_cgemm16<T, 0, 0><<<g, 256, 0, st>>>(M, N, K, A, lda, B, ldb, epi, kchunk, ws, tri);
+  else if (ta == 1 && tb == 0) k_cgemm16<T, 1, 0><<<g, 256, 0, st>>>(M, N, K, A, lda, B, ldb, epi, kchunk, ws, tri);
+  else if (ta == 0 && tb == 1) k_cgemm16<T, 0, 1><<<g, 256, 0, st>>>(M, N, K, A, lda, B, ldb, epi, kchunk, ws, tri);
+  else k_cgemm16<T, 1, 1><<<g, 256, 0, st>>>(M, N, K, A, lda, B, ldb, epi, kchunk, ws, tri);
+  count_launch();
+  if (nsplit > 1) {
+    const int64_t tot = (int64_t)M * N;
+    k_splitk_reduce<T><<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(M, N, nsplit, ws, epi, tri); count_launch();
+  }
+  return cudaGetLastError();
+}
+
+template <typename T>
 cudaError_t launch_cgemm(int ta, int tb, int M, int N, int K, const cplx<T>* A, int64_t lda,
                          const cplx<T>* B, int64_t ldb, const Epi<T>& epi, int nsplit, cplx<T>* ws,
                          cudaStream_t st, int tri) {
@@ -290,15 +317,8 @@ cudaError_t launch_cgemm(int ta, int tb, int M, int N, int K, const cplx<T>* A, 
   // without split: 16 x 16 tiles while the 64 x 64 ones do not give every SM one.  FP64: always the
   // better there; FP32 reuses an operand from registers 4 times in the large tile, which pays from
   // about 16 tiles on
-  if (nsplit == 1 && K > 0 && tm * tn < (sizeof(T) == 8 ? 152 : 16)) {
-    const dim3 g((M + 15) / 16, (N + 15) / 16);
-    if (ta == 0 && tb == 0) k_cgemm16<T, 0, 0><<<g, 256, 0, st>>>(M, N, K, A, lda, B, ldb, epi, tri);
-    else if (ta == 1 && tb == 0) k_cgemm16<T, 1, 0><<<g, 256, 0, st>>>(M, N, K, A, lda, B, ldb, epi, tri);
-    else if (ta == 0 && tb == 1) k_cgemm16<T, 0, 1><<<g, 256, 0, st>>>(M, N, K, A, lda, B, ldb, epi, tri);
-    else k_cgemm16<T, 1, 1><<<g, 256, 0, st>>>(M, N, K, A, lda, B, ldb, epi, tri);
-    count_launch();
-    return cudaGetLastError();
-  }
+  if (nsplit == 1 && K > 0 && tm * tn < (sizeof(T) == 8 ? 152 : 16))
+    return launch_cgemm16<T>(ta, tb, M, N, K, A, lda, B, ldb, epi, 1, nullptr, st, tri);
   dim3 grid(tm, tn, nsplit);
   if (tri == GEMM_LOWER_OUT) grid = dim3(tm * (tm + 1) / 2, 1, nsplit);
   if (ta == 0 && tb == 0) k_cgemm<T, 0, 0><<<grid, 256, 0, st>>>(M, N, K, A, lda, B, ldb, epi, kchunk, ws, tri);
@@ -342,6 +362,8 @@ cudaError_t launch_dblock(int nproj, int nband, const T* D, const int* blk0, con
   return cudaGetLastError();
 }
 
+template cudaError_t launch_cgemm16<double>(int, int, int, int, int, const double2*, int64_t, const double2*,
+                                            int64_t, const Epi<double>&, int, double2*, cudaStream_t, int);
 template cudaError_t launch_cgemm<double>(int, int, int, int, int, const double2*, int64_t, const double2*,
                                           int64_t, const Epi<double>&, int, double2*, cudaStream_t, int);
 template cudaError_t launch_cgemm<float>(int, int, int, int, int, const float2*, int64_t, const float2*,

@@ -411,6 +411,16 @@ int zgemm(pw_ctx* ctx, int ta, int tb, int M, int N, int K, const double2* A, in
     CU_TRY(launch_cgemm<double>(ta, tb, M, N, K, A, lda, B, ldb, e, dfma_ns, dfma_ws, st, tri), where);
     return PW_OK;
   }
+  // Small products: slicing two operands and one chunk of the digit GEMM take 75 us (8 x 16 x 925 as
+  // much as 136 x 32 x 14771), the FP64 pipe 29 us for 2^22 complex products over all SMs
+  // (the failure-path hook asks for a digit GEMM of any size)
+  if ((double)M * N * K < (double)(1 << 22) && !ctx->test_wait_expiry) {
+    const int tiles = ((M + 15) / 16) * ((N + 15) / 16);
+    const int ns = std::max(1, std::min((2 * 152) / tiles, K / 32));
+    WS(part, double2, WS_OZPART, (size_t)(ns > 1 ? ns : 0) * M * N + 1);
+    CU_TRY(launch_cgemm16<double>(ta, tb, M, N, K, A, lda, B, ldb, e, ns, part, st, tri), where);
+    return PW_OK;
+  }
   PW_TRY(ensure_err_flag(ctx));
   const int lower = (tri == GEMM_LOWER_OUT);
   oz::Digits Ad{nullptr, 2 * M, 2 * K, oz::digit_pitch(2 * K), 0, nullptr, digits};

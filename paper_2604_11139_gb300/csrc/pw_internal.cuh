@@ -228,6 +228,11 @@ cudaError_t launch_cgemm(int ta, int tb, int M, int N, int K, const cplx<T>* A, 
                          const cplx<T>* B, int64_t ldb, const Epi<T>& epi, int nsplit, cplx<T>* ws,
                          cudaStream_t st, int tri = GEMM_FULL);
 
+// the same product in 16 x 16 tiles, K in at most nsplit parts (ws: nsplit*M*N complex when > 1)
+template <typename T>
+cudaError_t launch_cgemm16(int ta, int tb, int M, int N, int K, const cplx<T>* A, int64_t lda, const cplx<T>* B,
+                           int64_t ldb, const Epi<T>& epi, int nsplit, cplx<T>* ws, cudaStream_t st, int tri);
+
 // real block-diagonal (or dense) D times complex C: Z = D C (nproj x nband)
 template <typename T>
 cudaError_t launch_dblock(int nproj, int nband, const T* D, const int* blk0, const int* blklen,
