@@ -17,9 +17,9 @@
 // (FP64 kernels 4.4e-16 to 5.2e-16), random, decaying, single-component and in-phase bands alike.
 //
 // What bounds them: issue of the integer instructions (half of the slots at 16 warps per SM, 42%
-// of the ALU pipe); the conversions to and from FP64 take a fifth of the FP64 pipe.  Radices and lengths are run-time values (a switch around
-// a stage, uniform in the CTA): one set of kernels covers every two-stage length, and the index
-// arithmetic is small beside 64-bit butterflies.
+// of the ALU pipe); the conversions to and from FP64 take a fifth of the FP64 pipe.  Radices and
+// lengths are run-time values (a switch around a stage, uniform in the CTA): one set of kernels
+// covers every two-stage length, and the index arithmetic is small beside 64-bit butterflies.
 //
 // Scales.  A line's inputs are multiplied by 2^(B - E), E the exponent of its largest component,
 // and rounded to integers |re|, |im| <= 2^B.  A radix-R stage grows the modulus by at most R; a
@@ -108,6 +108,17 @@ __device__ __forceinline__ ll mulv(int al, int ah, int vl, int vh) {
   ll m = madw(al, vh, kRound32);
   m = madw(ah, vl, m);
   return madw(ah, vh, sext_hi(m));
+}
+
+// round(Re(conj(a) b) / 2^64)
+__device__ __forceinline__ ll dot64(fc a, fc b) {
+  const int axl = lo32(a.x), axh = hi32(a.x), ayl = lo32(a.y), ayh = hi32(a.y);
+  const int bxl = lo32(b.x), bxh = hi32(b.x), byl = lo32(b.y), byh = hi32(b.y);
+  ll m = madw(axl, bxh, kRound32);
+  m = madw(axh, bxl, m);
+  m = madw(ayl, byh, m);
+  m = madw(ayh, byl, m);
+  return madw(ayh, byh, madw(axh, bxh, sext_hi(m)));
 }
 
 // ---- small DFTs: y_m = sum_k x_k exp(S 2 pi i k m / R) ------------------------------------
@@ -258,7 +269,8 @@ constexpr int kNan = 1 << 30;  // Out::k of a line with a component that is not 
 struct In {
   int add;       // (bits - E) << 20
   unsigned thr;  // high words below it (|x| 2^(bits - E) < 1/4, or no normal number) give 0
-  __device__ __forceinline__ In(int E, int bits) : add((bits - E) * (1 << 20)), thr((unsigned)max(1, E - bits + 1021) << 20) {}
+  __device__ __forceinline__ In(int E, int bits)
+      : add((bits - E) * (1 << 20)), thr((unsigned)max(1, E - bits + 1021) << 20) {}
   __device__ __forceinline__ ll operator()(double x) const {
     const int hi = __double2hiint(x);
     const bool z = ((unsigned)hi & 0x7fffffffu) < thr;
@@ -330,7 +342,10 @@ __device__ __forceinline__ void inv1(fc* col, int J, const Dim& d, In in, V vali
   for (int a = 0; a < R; ++a) {
     const int e = J + d.r2 * a;
     x[a] = valid(e) ? in(*reinterpret_cast<const double2*>(&col[e * PT])) : fc{0, 0};
-    if constexpr (NORM) *ss = madw((int)(x[a].x >> 32), (int)(x[a].x >> 32), madw((int)(x[a].y >> 32), (int)(x[a].y >> 32), *ss));
+    if constexpr (NORM) {
+      const int hx = (int)(x[a].x >> 32), hy = (int)(x[a].y >> 32);
+      *ss = madw(hx, hx, madw(hy, hy, *ss));
+    }
   }
   dft<+1, R>(x);
   col[J * PT] = quarter(x[0]);
@@ -447,10 +462,11 @@ __global__ void __launch_bounds__(kThreads, BIG ? 2 : 3) k_fx_zinv(const double2
 }
 
 template <bool BIG>
-__global__ void __launch_bounds__(kThreads, BIG ? 2 : 3) k_fx_zfwd(const double2* __restrict__ hb, int64_t hb_bs, SphereDev sp,
-                                                         Dim d, int n2, int bits, const double* __restrict__ kin,
-                                                         const double2* __restrict__ psi, int64_t ldpsi,
-                                                         double2* __restrict__ out, int64_t ldout) {
+__global__ void __launch_bounds__(kThreads, BIG ? 2 : 3) k_fx_zfwd(const double2* __restrict__ hb, int64_t hb_bs,
+                                                                   SphereDev sp, Dim d, int n2, int bits,
+                                                                   const double* __restrict__ kin,
+                                                                   const double2* __restrict__ psi, int64_t ldpsi,
+                                                                   double2* __restrict__ out, int64_t ldout) {
   extern __shared__ __align__(16) unsigned char smem[];
   fc* buf = reinterpret_cast<fc*>(smem);
   __shared__ unsigned rmax[32];
@@ -686,26 +702,29 @@ __global__ void __launch_bounds__(kThreads, BIG ? 2 : 3) k_fx_x(double2* __restr
 
 // ---- density: inverse x of a (and b), out[r] += sum_b w_b Re[conj(a) b] --------------------------
 // 32 lines per CTA and a share of the bands (blockIdx.y); the sums stay in shared memory until the
-// end and are added to the permuted grid atomically.  The products and sums are FP64: they take
-// about as long as the transform, on the other pipe.
+// end and are added to the permuted grid atomically.  The products are integers too, of the values
+// shifted up to 2^62 by what the line's 2-norm allows (|value| <= sqrt(np) times it): one conversion
+// and one FMA per point are left to the FP64 pipe, which was the bound with FP64 products.
 template <bool BIG>
 __global__ void __launch_bounds__(kThreads, BIG ? 2 : 3) k_fx_dens(const double2* __restrict__ hba,
                                                          const double2* __restrict__ hbb, int64_t hb_bs, int nb,
                                                          int bper, const double* __restrict__ wgt, int np, int nyz,
-                                                         Dim d, int bits, double* __restrict__ out_perm) {
+                                                         Dim d, int bits, int room,
+                                                         double* __restrict__ out_perm) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, n = d.n;
   fc* bufa = reinterpret_cast<fc*>(smem);
   fc* bufb = bufa + (hbb ? n * PT : 0);
   double* acc = reinterpret_cast<double*>(bufb + n * PT) + lane;  // [n][32]
   __shared__ unsigned red[2][kWarps][32];
+  __shared__ ll red2[2][kWarps][32];
   const int yz = blockIdx.x * 32 + lane;
   const bool live = yz < nyz;
   for (int e = w; e < n; e += kWarps) acc[e * 32] = 0.0;
   const int b_lo = blockIdx.y * bper, b_hi = min(nb, b_lo + bper);
 #pragma unroll 1
   for (int b = b_lo; b < b_hi; ++b) {
-    Out oa{0}, ob{0};
+    int ka = 0, kb = 0;  // exponents of a and b; kNan
 #pragma unroll 1
     for (int which = 0; which < (hbb ? 2 : 1); ++which) {
       const double2* pl = (which ? hbb : hba) + (int64_t)b * hb_bs + (live ? yz : 0);
@@ -720,17 +739,27 @@ __global__ void __launch_bounds__(kThreads, BIG ? 2 : 3) k_fx_dens(const double2
       mx = line_max(mx, red[which]);
       const int E = top_exp(mx);
       const In in(E, bits);
-      (which ? ob : oa).k = out_exp(mx, E - bits + 2);
+      (which ? kb : ka) = out_exp(mx, E - bits + 2);
+      ll ss = 0;
 #define FX_F(R)                                              \
   _Pragma("unroll 1") for (int J = w; J < d.r2; J += kWarps) \
-      inv1<R>(col, J, d, in, [&](int e) { return e < np; })
+      inv1<R, true>(col, J, d, in, [&](int e) { return e < np; }, &ss)
       FX_SWITCH(d.r1, FX_F)
 #undef FX_F
+      red2[which][w][lane] = ss;
     }
-    if (!hbb) ob = oa;
     __syncthreads();
+    auto shift = [&](int which) {
+      ll ss = 1;
+#pragma unroll
+      for (int i = 0; i < kWarps; ++i) ss += red2[which][i][lane];
+      return min(max((__clzll(ss) - room) >> 1, 0), 12);
+    };
+    const int ta = shift(0), tb = hbb ? shift(1) : ta;
+    if (!hbb) kb = ka;
+    const Out of{ka == kNan || kb == kNan ? kNan : ka + kb - ta - tb + 64};
     const double wb = wgt[b];
-    // the last stage of a (and b); with b, a's values go back to its line as FP64
+    // the last stage of a (and b); with b, a's values go back to its line
 #define FX_F(R)                                                                   \
   _Pragma("unroll 1") for (int blk = w; blk < d.r1; blk += kWarps) {              \
     fc y[R];                                                                      \
@@ -738,16 +767,16 @@ __global__ void __launch_bounds__(kThreads, BIG ? 2 : 3) k_fx_dens(const double2
       fc* ca = bufa + lane + blk * R * PT;                                        \
       _Pragma("unroll") for (int m = 0; m < R; ++m) y[m] = ca[m * PT];            \
       dft<+1, R>(y);                                                              \
-      _Pragma("unroll") for (int m = 0; m < R; ++m)                               \
-          *reinterpret_cast<double2*>(&ca[m * PT]) = oa(y[m]);                    \
+      _Pragma("unroll") for (int m = 0; m < R; ++m) ca[m * PT] = {y[m].x << ta, y[m].y << ta}; \
     }                                                                             \
     const fc* cb = bufb + lane + blk * R * PT;                                    \
     _Pragma("unroll") for (int m = 0; m < R; ++m) y[m] = cb[m * PT];              \
     dft<+1, R>(y);                                                                \
     _Pragma("unroll") for (int m = 0; m < R; ++m) {                               \
-      const double2 vb = ob(y[m]);                                                \
-      const double2 va = hbb ? *reinterpret_cast<const double2*>(&bufa[lane + (blk * R + m) * PT]) : vb; \
-      acc[(blk * R + m) * 32] += wb * (va.x * vb.x + va.y * vb.y);                \
+      const fc vb = {y[m].x << tb, y[m].y << tb};                                 \
+      const fc va = hbb ? bufa[lane + (blk * R + m) * PT] : vb;                   \
+      double* s = &acc[(blk * R + m) * 32];                                       \
+      *s = fma(wb, of(dot64(va, vb)), *s);                                        \
     }                                                                             \
   }
     FX_SWITCH(d.r2, FX_F)
@@ -760,17 +789,42 @@ __global__ void __launch_bounds__(kThreads, BIG ? 2 : 3) k_fx_dens(const double2
 }
 
 // ---- host -------------------------------------------------------------------------------
-Tw twiddle(long jm, long L) {
-  const long double ang = -2.0L * 3.14159265358979323846264338327950288L * (long double)jm / (long double)L;
-  const long double one = 4611686018427387904.0L;
+std::vector<Tw> twiddles(int L) {
+  // angle 2 pi k / L: octant 8 k / L, remainder r / L of pi / 4 (mirrored in odd octants), so the
+  // long double functions (software on some hosts) run once per remainder and below pi / 4 only
+  const long long one = 1ll << 62;
+  std::vector<long long> c(L + 1), s(L + 1);
+  std::vector<char> have(L + 1, 0);
   auto halves = [](long long v, int& lo, int& hi) {
     if ((int)(unsigned)(v & 0xffffffffll) == INT32_MIN) v += 1;  // keep -lo representable
     lo = (int)(unsigned)(v & 0xffffffffll);
     hi = (int)((v - lo) >> 32);
   };
-  Tw t;
-  halves(llroundl(cosl(ang) * one), t.xlo, t.xhi);
-  halves(llroundl(sinl(ang) * one), t.ylo, t.yhi);
+  std::vector<Tw> t(L);
+  for (int k = 0; k < L; ++k) {
+    const int o = (int)(8ll * k / L), r0 = (int)(8ll * k - (long long)o * L), r = (o & 1) ? L - r0 : r0;
+    if (!have[r]) {
+      const long double a = 0.78539816339744830961566084581987572L * (long double)r / (long double)L;
+      c[r] = llroundl(cosl(a) * (long double)one);
+      s[r] = llroundl(sinl(a) * (long double)one);
+      have[r] = 1;
+    }
+    // cos and sin of pi / 4 o' + a (o odd: pi / 4 (o + 1) - a)
+    const long long C = c[r], Sn = s[r];
+    long long x, y;
+    switch (o) {
+      case 0: x = C; y = Sn; break;
+      case 1: x = Sn; y = C; break;
+      case 2: x = -Sn; y = C; break;
+      case 3: x = -C; y = Sn; break;
+      case 4: x = -C; y = -Sn; break;
+      case 5: x = -Sn; y = -C; break;
+      case 6: x = Sn; y = -C; break;
+      default: x = C; y = -Sn; break;
+    }
+    halves(x, t[k].xlo, t[k].xhi);
+    halves(-y, t[k].ylo, t[k].yhi);  // exp(-i angle)
+  }
   return t;
 }
 
@@ -860,6 +914,11 @@ cudaError_t local_apply(const FftPlan& plan, const double2* tw, const SphereDev&
   return cudaGetLastError();
 }
 
+// The same for the density: the values, at most sqrt(np) 2^(x - 2 + t), stay below 2^62.
+static int room_dens(int np) {
+  return (int)ceil(64.0 - 2.0 * (62.0 + 2.0 - 0.5 * log2((double)np) - 32.0));
+}
+
 cudaError_t density(const FftPlan& plan, const double2* tw, const SphereDev& sp, const double2* a, const double2* b,
                     int64_t ld, int nband, const double* w_dev, double* out_perm, double2* hb, int band_batch,
                     cudaStream_t st) {
@@ -870,7 +929,7 @@ cudaError_t density(const FftPlan& plan, const double2* tw, const SphereDev& sp,
   const size_t line = sizeof(fc) * PT;
   const size_t smz = line * dz.n, smy = line * dy.n + sizeof(int) * dy.n;
   const size_t smx = line * dx.n * (b ? 2 : 1) + sizeof(double) * 32 * dx.n;
-  if (smx > 224 * 1024) return cudaErrorNotSupported;
+  if (smx > 220 * 1024) return cudaErrorNotSupported;  // 6 KB more are static
   cudaError_t e;
   auto attr = [&](const void* f, size_t sm) {
     return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
@@ -892,7 +951,7 @@ cudaError_t density(const FftPlan& plan, const double2* tw, const SphereDev& sp,
     const int bper = (nb + splits - 1) / splits;
     splits = (nb + bper - 1) / bper;
     (big(dx) ? k_fx_dens<true> : k_fx_dens<false>)<<<dim3(gx, splits), kThreads, smx, st>>>(hb, hbb, hb_bs, nb, bper, w_dev + b0, sp.nplane, nyz, dx, bx,
-                                                       out_perm); count_launch();
+                                                       room_dens(sp.nplane), out_perm); count_launch();
   }
   return cudaGetLastError();
 }

@@ -23,8 +23,8 @@ struct Tw {
 };
 static_assert(sizeof(Tw) == sizeof(double2), "the fixed-point table follows the FP64 one in memory");
 
-// The table entry of angle -2 pi jm / L (0 <= jm < L), from long double sine and cosine.
-Tw twiddle(long jm, long L);
+// exp(-2 pi i k / L) for k < L, from long double sine and cosine.
+std::vector<Tw> twiddles(int L);
 
 // Whether the passes cover the box: every length with a two-stage plan, up to 256.
 bool covers(const FftPlan& plan);

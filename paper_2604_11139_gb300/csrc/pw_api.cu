@@ -12,6 +12,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <map>
 #include <new>
 #include <type_traits>
 #include <vector>
@@ -1438,18 +1439,21 @@ int create_impl(const pw_problem_desc* d, void* stream, pw_ctx** out) {
   // twiddles e^{-2 pi i j m / L}; the fixed-point table of the complex128 passes has the same layout
   std::vector<double2> tw;
   std::vector<fx::Tw> twf;
+  std::map<int, std::vector<fx::Tw>> wfix;  // by stage length
   for (int dd = 0; dd < 3; ++dd) {
     FftDim& f = ctx->plan.d[dd];
     f.tw_base = (int)tw.size();
     for (int s = 0; s < f.nst; ++s) {
       f.tw_off[s] = (int)tw.size();
       const int L = f.L[s], r = f.radix[s], q = L / r;
+      auto& wf = wfix[L];
+      if (wf.empty()) wf = fx::twiddles(L);
       for (int j = 0; j < q; ++j)
         for (int m = 1; m < r; ++m) {
           const long jm = ((long)j * m) % L;
           const double ang = -2.0 * kPi * (double)jm / (double)L;
           tw.push_back(make_double2(cos(ang), sin(ang)));
-          twf.push_back(fx::twiddle(jm, L));
+          twf.push_back(wf[jm]);
         }
     }
     f.tw_count = (int)tw.size() - f.tw_base;

@@ -121,3 +121,18 @@ def test_density(box, two):
         ref += w[i] * (ga.conj() * gb).real
         size += w[i] * abs(ga) * abs(gb)
     assert float(np.sqrt((abs(rho - ref) ** 2).sum() / (size ** 2).sum())) < TOL
+
+
+@pytest.mark.parametrize("kind", ["normal", "single", "peak"])
+def test_density_of_uneven_lines(kind):
+    box = (45, 50, 54)
+    rng = np.random.default_rng(11)
+    ctx, at, kin = make(box, rng.standard_normal(box))
+    a = block(rng, kind, kin)
+    rho = ctx.density_grad(torch.from_numpy(a).cuda(), [1.0, -0.5, 2.0]).cpu().numpy().reshape(box)
+    ref, size = np.zeros(box, np.longdouble), np.zeros(box, np.longdouble)
+    for i, w in enumerate((1.0, -0.5, 2.0)):
+        g = abs(grid(box, at, a[i])) ** 2
+        ref += w * g
+        size += abs(w) * g
+    assert float(np.sqrt((abs(rho - ref) ** 2).sum() / (size ** 2).sum())) < TOL
