@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(kThreads) k_fl_zfwd(const C* __restrict__ hb, 
       if constexpr (!REC) {
         o[gg] = make_float2(k * yy.x + v.x, k * yy.y + v.y);
       } else {
-        const C pz = rec.pz[(int64_t)b * rec.ldpz + gg];
+        const C pz = rec.pz ? rec.pz[(int64_t)b * rec.ldpz + gg] : make_float2(0.f, 0.f);
         C t = make_float2(ra * (k * yy.x + v.x + pz.x - rs * yy.x), ra * (k * yy.y + v.y + pz.y - rs * yy.y));
         if (rec.ykm1) {
           const C ym = rec.ykm1[(int64_t)b * rec.ldykm1 + gg];

@@ -2155,7 +2155,7 @@ __device__ __forceinline__ void plane_fwd_wg_item(int p, int b, const cplx<T>* _
       if constexpr (!REC) {
         o[gg] = mk<C>(k * yy.x + v.x, k * yy.y + v.y);
       } else {
-        const C pz = ((const C*)rec.pz)[(int64_t)b * rec.ldpz + gg];
+        const C pz = rec.pz ? ((const C*)rec.pz)[(int64_t)b * rec.ldpz + gg] : czero<C>();
         C r = mk<C>(ra * (k * yy.x + v.x + pz.x - rs * yy.x), ra * (k * yy.y + v.y + pz.y - rs * yy.y));
         if (rec.ykm1) {
           const C ym = ((const C*)rec.ykm1)[(int64_t)b * rec.ldykm1 + gg];
@@ -2622,7 +2622,7 @@ __global__ void __launch_bounds__(PlaneR<N2, N3, TW>::THREADS) k_plane_fwd_rs(co
       if constexpr (!REC) {
         o[gg] = mk<C>(k * yy.x + v.x, k * yy.y + v.y);
       } else {
-        const C pz = ((const C*)rec.pz)[(int64_t)b * rec.ldpz + gg];
+        const C pz = rec.pz ? ((const C*)rec.pz)[(int64_t)b * rec.ldpz + gg] : czero<C>();
         C r = mk<C>(ra * (k * yy.x + v.x + pz.x - rs * yy.x), ra * (k * yy.y + v.y + pz.y - rs * yy.y));
         if (rec.ykm1) {
           const C ym = ((const C*)rec.ykm1)[(int64_t)b * rec.ldykm1 + gg];
@@ -3015,7 +3015,7 @@ cudaError_t launch_local_apply_rec(const FftPlan& plan, const float2* tw, const 
     prof_end(prof, PW_PROF_XLINE);
     prof_begin(prof, PW_PROF_PLANE_FWD);
     Pass3Rec r = rec;
-    r.pz = rec.pz + b0 * rec.ldpz;
+    if (rec.pz) r.pz = rec.pz + b0 * rec.ldpz;
     if (rec.ykm1) r.ykm1 = rec.ykm1 + b0 * rec.ldykm1;
     if (rec.split) r.split = (__nv_bfloat16*)rec.split + b0 * rec.split_ld;
     e = prs ? plane_rs<T>(1, psi + b0 * ldpsi, ldpsi, hb, hb_bs, sp, plan, tw, kin, out + b0 * ldout, ldout, nb, st,

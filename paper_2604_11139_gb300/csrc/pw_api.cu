@@ -612,6 +612,10 @@ int filter_impl(pw_ctx* ctx, cplx<T>* psi, int64_t ldpsi, int nband, int degree,
   const int64_t ld[3] = {ldpsi, npw, npw};
   const double cc = 0.5 * (b + a), e = 0.5 * (b - a);
   constexpr bool kMixed = std::is_same<T, float>::value;
+  // projector-space products in complex64: K in two parts where the 64 x 64 tiles alone leave SMs
+  // without one (864 x 512 x 864, 112 tiles: 128 -> 109 us), not below 16 tiles (see launch_cgemm)
+  const int ptiles = ((np + 63) / 64) * ((nband + 63) / 64);
+  const int nsq = kMixed && ptiles >= 16 && ptiles < 152 ? std::min(ns, std::max(1, std::min(304 / ptiles, np / 128))) : 1;
   __nv_bfloat16* ys = nullptr;
   int64_t ys_ps = 0;  // piece stride of the bf16 pieces; kp1 is known once the operands of P exist
   if (kMixed && np > 0) {
@@ -643,7 +647,7 @@ int filter_impl(pw_ctx* ctx, cplx<T>* psi, int64_t ldpsi, int nband, int degree,
     ce.ldy2 = np;
     ce.dev_ce = dev_ce;
     ce.first = (k == 0);
-    PW_TRY(cg<T>(ctx, 0, 0, np, nband, np, Prec<T>::B(ctx), np, Z, np, ce, 1, spl, st, GEMM_FULL,
+    PW_TRY(cg<T>(ctx, 0, 0, np, nband, np, Prec<T>::B(ctx), np, Z, np, ce, nsq, spl, st, GEMM_FULL,
                  "projector-space recurrence"));
     return PW_OK;
   };
@@ -709,14 +713,30 @@ int filter_impl(pw_ctx* ctx, cplx<T>* psi, int64_t ldpsi, int nband, int degree,
     C* dst = buf[(k + 1) % 3];
     const int64_t ldc = ld[k % 3], ldp = ld[(k + 2) % 3], ldd = ld[(k + 1) % 3];
     const T alpha = (T)(k == 0 ? 1.0 / e : 2.0 / e);
-    // W = (T + V) Y_k
-    CU_TRY(launch_local_apply<T>(ctx->plan, Prec<T>::tw(ctx), ctx->sp, Prec<T>::vp(ctx), Prec<T>::kin(ctx), cur,
-                                 ldc, nband, dst, ldd, hb, bb, st, ctx), "filter local");
+    // W = (T + V) Y_k; with Q and a kernel for it, pass 3 also writes the bf16 pieces of W that the
+    // projection takes (512 bands on 120^3, 12 steps: the pass over W took 4.6 ms, pass 3 2.2 ms longer)
+    bool pieces_done = false;
+    if constexpr (kMixed) {
+      if (shadow && local_apply_rec_supported(ctx->plan, ctx)) {
+        Pass3Rec rec{};
+        rec.alpha = 1.f;
+        rec.split = ys;
+        rec.split_ld = ctx->kp1;
+        rec.split_piece_stride = ys_ps;
+        rec.pieces = ctx->tc_pieces;
+        CU_TRY(launch_local_apply_rec(ctx->plan, ctx->tw32, ctx->sp, ctx->vperm32, ctx->kin32, (const float2*)cur, ldc,
+                                      nband, (float2*)dst, ldd, (float2*)hb, bb, st, ctx, rec), "filter local + split");
+        pieces_done = true;
+      }
+    }
+    if (!pieces_done)
+      CU_TRY(launch_local_apply<T>(ctx->plan, Prec<T>::tw(ctx), ctx->sp, Prec<T>::vp(ctx), Prec<T>::kin(ctx), cur,
+                                   ldc, nband, dst, ldd, hb, bb, st, ctx), "filter local");
     if (kMixed && np > 0) {
       {
         ProfScope ps(ctx, PW_PROF_GEMM_PROJ);
         if (shadow) {
-          PW_TRY(tc_split_into(ctx, (const float2*)dst, ldd, npw, nband, ctx->kp1, ys_ps, ys));
+          if (!pieces_done) PW_TRY(tc_split_into(ctx, (const float2*)dst, ldd, npw, nband, ctx->kp1, ys_ps, ys));
           PW_TRY(tc_project(ctx, ys, nband, (float2*)Cw));  // P^dagger W; C_k from the recurrence
         } else {
           PW_TRY(tc_project(ctx, ys, nband, (float2*)Cm));
@@ -728,8 +748,8 @@ int filter_impl(pw_ctx* ctx, cplx<T>* psi, int64_t ldpsi, int nband, int degree,
         if (!ctx->has_q) {
           CU_TRY(launch_dblock<T>(np, nband, Prec<T>::D(ctx), ctx->blk0, ctx->blklen, Cm, np, Z, np, st), "filter D");
         } else {
-          PW_TRY(cg<T>(ctx, 0, 0, np, nband, np, Prec<T>::E(ctx), np, Crot(k), np, epi<T>(EPI_STORE, Z, np), 1, spl, st, GEMM_FULL, "filter E C"));
-          PW_TRY(cg<T>(ctx, 0, 0, np, nband, np, Prec<T>::K(ctx), np, Cw, np, epi<T>(EPI_ACCUM, Z, np, (T)-1), 1, spl, st, GEMM_FULL, "filter K Cw"));
+          PW_TRY(cg<T>(ctx, 0, 0, np, nband, np, Prec<T>::E(ctx), np, Crot(k), np, epi<T>(EPI_STORE, Z, np), nsq, spl, st, GEMM_FULL, "filter E C"));
+          PW_TRY(cg<T>(ctx, 0, 0, np, nband, np, Prec<T>::K(ctx), np, Cw, np, epi<T>(EPI_ACCUM, Z, np, (T)-1), nsq, spl, st, GEMM_FULL, "filter K Cw"));
         }
         PW_TRY(tc_split(ctx, (const float2*)Z, np, np, nband, ctx->kp2, WS_ZSPLIT, &zs));
       }

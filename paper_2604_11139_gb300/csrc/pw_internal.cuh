@@ -184,7 +184,7 @@ cudaError_t launch_local_apply(const FftPlan& plan, const cplx<T>* tw, const Sph
 
 // Recurrence step fused into FFT pass 3 (complex64, S = I):
 //   y_{k+1} = alpha (kin y_k + (V y_k) + pz - shift y_k) - beta y_{k-1}
-// pz = P D P^dagger y_k from the back-projection GEMM (ld ldpz); ykm1 may be NULL; with
+// pz = P D P^dagger y_k from the back-projection GEMM (ld ldpz), NULL for none; ykm1 may be NULL; with
 // dev_ce, shift = c and alpha = (first ? 1 : 2) / e are read from the device.  split (may be
 // NULL) receives the bf16 pieces of y_{k+1}: piece p of band b, real row r (2g: Re, 2g+1: Im)
 // at split[p * split_piece_stride + b * split_ld + r].
