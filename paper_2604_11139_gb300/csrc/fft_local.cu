@@ -2807,7 +2807,7 @@ cudaError_t launch_local_apply(const FftPlan& plan, const cplx<T>* tw, const Sph
                                cudaStream_t st, ::pw_ctx* prof) {
   if (nband <= 0) return cudaSuccess;
   if constexpr (std::is_same<T, double>::value) {
-    if (fx::covers(plan))
+    if (fx::covers(plan) && !(prof && prof->keep64))
       return fx::local_apply(plan, tw, sp, vperm, kin, psi, ldpsi, nband, out, ldout, hb, band_batch, st, prof);
   }
   const int cz = pick_cz(plan.n[2]);

@@ -88,62 +88,62 @@ template <typename C, int S> __device__ __forceinline__ void dft5(C* x) {
   x[1] = bf_add_muli<S>(a1, u1); x[4] = bf_sub_muli<S>(a1, u1);
   x[2] = bf_add_muli<S>(a2, u2); x[3] = bf_sub_muli<S>(a2, u2);
 }
-// exp(-2 pi i m / R) for the composite in-register radices.
+// exp(-2 pi i m / R) for the composite in-register radices: cos and sin of the FP64 angle.
 // Offsets: R=6: 0, 9: 6, 10: 15, 12: 25, 15: 37, 16: 52.
 static __constant__ double2 c_wtab64[68] = {
-    {1.0, 0.0}, {0.5, -0.8660254037844386}, {-0.5, -0.8660254037844386}, {-1.0, 0.0}, {-0.5, 0.8660254037844386},
-    {0.5, 0.8660254037844386}, {1.0, 0.0}, {0.766044443118978, -0.6427876096865394},
-    {0.17364817766693036, -0.984807753012208}, {-0.5, -0.8660254037844386},
-    {-0.9396926207859084, -0.3420201433256687}, {-0.9396926207859084, 0.3420201433256687},
-    {-0.5, 0.8660254037844386}, {0.17364817766693036, 0.984807753012208}, {0.766044443118978, 0.6427876096865394},
-    {1.0, 0.0}, {0.8090169943749475, -0.5877852522924731}, {0.30901699437494745, -0.9510565162951535},
-    {-0.30901699437494745, -0.9510565162951535}, {-0.8090169943749475, -0.5877852522924731}, {-1.0, 0.0},
-    {-0.8090169943749475, 0.5877852522924731}, {-0.30901699437494745, 0.9510565162951535},
-    {0.30901699437494745, 0.9510565162951535}, {0.8090169943749475, 0.5877852522924731}, {1.0, 0.0},
-    {0.8660254037844386, -0.5}, {0.5, -0.8660254037844386}, {0.0, -1.0}, {-0.5, -0.8660254037844386},
-    {-0.8660254037844386, -0.5}, {-1.0, 0.0}, {-0.8660254037844386, 0.5}, {-0.5, 0.8660254037844386}, {0.0, 1.0},
-    {0.5, 0.8660254037844386}, {0.8660254037844386, 0.5}, {1.0, 0.0}, {0.9135454576426009, -0.4067366430758002},
-    {0.6691306063588582, -0.7431448254773942}, {0.30901699437494745, -0.9510565162951535},
-    {-0.10452846326765347, -0.9945218953682733}, {-0.5, -0.8660254037844386},
-    {-0.8090169943749475, -0.5877852522924731}, {-0.9781476007338057, -0.20791169081775934},
-    {-0.9781476007338057, 0.20791169081775934}, {-0.8090169943749475, 0.5877852522924731},
-    {-0.5, 0.8660254037844386}, {-0.10452846326765347, 0.9945218953682733},
-    {0.30901699437494745, 0.9510565162951535}, {0.6691306063588582, 0.7431448254773942},
-    {0.9135454576426009, 0.4067366430758002}, {1.0, 0.0}, {0.9238795325112867, -0.3826834323650898},
-    {0.7071067811865476, -0.7071067811865476}, {0.3826834323650898, -0.9238795325112867}, {0.0, -1.0},
-    {-0.3826834323650898, -0.9238795325112867}, {-0.7071067811865476, -0.7071067811865476},
-    {-0.9238795325112867, -0.3826834323650898}, {-1.0, 0.0}, {-0.9238795325112867, 0.3826834323650898},
-    {-0.7071067811865476, 0.7071067811865476}, {-0.3826834323650898, 0.9238795325112867}, {0.0, 1.0},
-    {0.3826834323650898, 0.9238795325112867}, {0.7071067811865476, 0.7071067811865476},
-    {0.9238795325112867, 0.3826834323650898},
+    {1.0, -0.0}, {0.5000000000000001, -0.8660254037844386}, {-0.4999999999999998, -0.8660254037844387},
+    {-1.0, -1.2246467991473532e-16}, {-0.5000000000000004, 0.8660254037844384},
+    {0.5000000000000001, 0.8660254037844386}, {1.0, -0.0}, {0.766044443118978, -0.6427876096865393},
+    {0.17364817766693041, -0.984807753012208}, {-0.4999999999999998, -0.8660254037844387},
+    {-0.9396926207859083, -0.3420201433256689}, {-0.9396926207859084, 0.34202014332566866},
+    {-0.5000000000000004, 0.8660254037844384}, {0.17364817766692997, 0.9848077530122081},
+    {0.7660444431189778, 0.6427876096865396}, {1.0, -0.0}, {0.8090169943749475, -0.5877852522924731},
+    {0.30901699437494745, -0.9510565162951535}, {-0.30901699437494734, -0.9510565162951536},
+    {-0.8090169943749473, -0.5877852522924732}, {-1.0, -1.2246467991473532e-16},
+    {-0.8090169943749476, 0.587785252292473}, {-0.30901699437494756, 0.9510565162951535},
+    {0.30901699437494723, 0.9510565162951536}, {0.8090169943749473, 0.5877852522924734}, {1.0, -0.0},
+    {0.8660254037844387, -0.49999999999999994}, {0.5000000000000001, -0.8660254037844386},
+    {6.123233995736766e-17, -1.0}, {-0.4999999999999998, -0.8660254037844387},
+    {-0.8660254037844387, -0.49999999999999994}, {-1.0, -1.2246467991473532e-16},
+    {-0.8660254037844388, 0.4999999999999997}, {-0.5000000000000004, 0.8660254037844384},
+    {-1.8369701987210297e-16, 1.0}, {0.5000000000000001, 0.8660254037844386},
+    {0.8660254037844384, 0.5000000000000004}, {1.0, -0.0}, {0.9135454576426009, -0.40673664307580015},
+    {0.6691306063588582, -0.7431448254773941}, {0.30901699437494745, -0.9510565162951535},
+    {-0.10452846326765333, -0.9945218953682734}, {-0.4999999999999998, -0.8660254037844387},
+    {-0.8090169943749473, -0.5877852522924732}, {-0.9781476007338057, -0.20791169081775931},
+    {-0.9781476007338057, 0.20791169081775907}, {-0.8090169943749476, 0.587785252292473},
+    {-0.5000000000000004, 0.8660254037844384}, {-0.10452846326765423, 0.9945218953682733},
+    {0.30901699437494723, 0.9510565162951536}, {0.6691306063588585, 0.743144825477394},
+    {0.913545457642601, 0.40673664307580015}, {1.0, -0.0}, {0.9238795325112867, -0.3826834323650898},
+    {0.7071067811865476, -0.7071067811865475}, {0.38268343236508984, -0.9238795325112867},
+    {6.123233995736766e-17, -1.0}, {-0.3826834323650897, -0.9238795325112867},
+    {-0.7071067811865475, -0.7071067811865476}, {-0.9238795325112867, -0.3826834323650899},
+    {-1.0, -1.2246467991473532e-16}, {-0.9238795325112868, 0.38268343236508967},
+    {-0.7071067811865477, 0.7071067811865475}, {-0.38268343236509034, 0.9238795325112865},
+    {-1.8369701987210297e-16, 1.0}, {0.38268343236509, 0.9238795325112866},
+    {0.7071067811865474, 0.7071067811865477}, {0.9238795325112865, 0.3826834323650904},
 };
 static __constant__ float2 c_wtab32[68] = {
-    {1.0f, 0.0f}, {0.5f, -0.8660254037844386f}, {-0.5f, -0.8660254037844386f}, {-1.0f, 0.0f},
-    {-0.5f, 0.8660254037844386f}, {0.5f, 0.8660254037844386f}, {1.0f, 0.0f},
-    {0.766044443118978f, -0.6427876096865394f}, {0.17364817766693036f, -0.984807753012208f},
-    {-0.5f, -0.8660254037844386f}, {-0.9396926207859084f, -0.3420201433256687f},
-    {-0.9396926207859084f, 0.3420201433256687f}, {-0.5f, 0.8660254037844386f},
-    {0.17364817766693036f, 0.984807753012208f}, {0.766044443118978f, 0.6427876096865394f}, {1.0f, 0.0f},
-    {0.8090169943749475f, -0.5877852522924731f}, {0.30901699437494745f, -0.9510565162951535f},
-    {-0.30901699437494745f, -0.9510565162951535f}, {-0.8090169943749475f, -0.5877852522924731f}, {-1.0f, 0.0f},
-    {-0.8090169943749475f, 0.5877852522924731f}, {-0.30901699437494745f, 0.9510565162951535f},
-    {0.30901699437494745f, 0.9510565162951535f}, {0.8090169943749475f, 0.5877852522924731f}, {1.0f, 0.0f},
-    {0.8660254037844386f, -0.5f}, {0.5f, -0.8660254037844386f}, {0.0f, -1.0f}, {-0.5f, -0.8660254037844386f},
-    {-0.8660254037844386f, -0.5f}, {-1.0f, 0.0f}, {-0.8660254037844386f, 0.5f}, {-0.5f, 0.8660254037844386f},
-    {0.0f, 1.0f}, {0.5f, 0.8660254037844386f}, {0.8660254037844386f, 0.5f}, {1.0f, 0.0f},
-    {0.9135454576426009f, -0.4067366430758002f}, {0.6691306063588582f, -0.7431448254773942f},
-    {0.30901699437494745f, -0.9510565162951535f}, {-0.10452846326765347f, -0.9945218953682733f},
-    {-0.5f, -0.8660254037844386f}, {-0.8090169943749475f, -0.5877852522924731f},
-    {-0.9781476007338057f, -0.20791169081775934f}, {-0.9781476007338057f, 0.20791169081775934f},
-    {-0.8090169943749475f, 0.5877852522924731f}, {-0.5f, 0.8660254037844386f},
-    {-0.10452846326765347f, 0.9945218953682733f}, {0.30901699437494745f, 0.9510565162951535f},
-    {0.6691306063588582f, 0.7431448254773942f}, {0.9135454576426009f, 0.4067366430758002f}, {1.0f, 0.0f},
-    {0.9238795325112867f, -0.3826834323650898f}, {0.7071067811865476f, -0.7071067811865476f},
-    {0.3826834323650898f, -0.9238795325112867f}, {0.0f, -1.0f}, {-0.3826834323650898f, -0.9238795325112867f},
-    {-0.7071067811865476f, -0.7071067811865476f}, {-0.9238795325112867f, -0.3826834323650898f}, {-1.0f, 0.0f},
-    {-0.9238795325112867f, 0.3826834323650898f}, {-0.7071067811865476f, 0.7071067811865476f},
-    {-0.3826834323650898f, 0.9238795325112867f}, {0.0f, 1.0f}, {0.3826834323650898f, 0.9238795325112867f},
-    {0.7071067811865476f, 0.7071067811865476f}, {0.9238795325112867f, 0.3826834323650898f},
+    {1.f, -0.f}, {0.5f, -0.866025388f}, {-0.5f, -0.866025388f}, {-1.f, -1.22464685e-16f}, {-0.5f, 0.866025388f},
+    {0.5f, 0.866025388f}, {1.f, -0.f}, {0.766044438f, -0.642787635f}, {0.173648179f, -0.98480773f},
+    {-0.5f, -0.866025388f}, {-0.939692616f, -0.342020154f}, {-0.939692616f, 0.342020154f}, {-0.5f, 0.866025388f},
+    {0.173648179f, 0.98480773f}, {0.766044438f, 0.642787635f}, {1.f, -0.f}, {0.809017003f, -0.587785244f},
+    {0.309017003f, -0.95105654f}, {-0.309017003f, -0.95105654f}, {-0.809017003f, -0.587785244f},
+    {-1.f, -1.22464685e-16f}, {-0.809017003f, 0.587785244f}, {-0.309017003f, 0.95105654f},
+    {0.309017003f, 0.95105654f}, {0.809017003f, 0.587785244f}, {1.f, -0.f}, {0.866025388f, -0.5f},
+    {0.5f, -0.866025388f}, {6.12323426e-17f, -1.f}, {-0.5f, -0.866025388f}, {-0.866025388f, -0.5f},
+    {-1.f, -1.22464685e-16f}, {-0.866025388f, 0.5f}, {-0.5f, 0.866025388f}, {-1.83697015e-16f, 1.f},
+    {0.5f, 0.866025388f}, {0.866025388f, 0.5f}, {1.f, -0.f}, {0.91354543f, -0.406736642f},
+    {0.669130623f, -0.74314481f}, {0.309017003f, -0.95105654f}, {-0.104528464f, -0.994521916f},
+    {-0.5f, -0.866025388f}, {-0.809017003f, -0.587785244f}, {-0.978147626f, -0.207911685f},
+    {-0.978147626f, 0.207911685f}, {-0.809017003f, 0.587785244f}, {-0.5f, 0.866025388f},
+    {-0.104528464f, 0.994521916f}, {0.309017003f, 0.95105654f}, {0.669130623f, 0.74314481f},
+    {0.91354543f, 0.406736642f}, {1.f, -0.f}, {0.923879504f, -0.382683426f}, {0.707106769f, -0.707106769f},
+    {0.382683426f, -0.923879504f}, {6.12323426e-17f, -1.f}, {-0.382683426f, -0.923879504f},
+    {-0.707106769f, -0.707106769f}, {-0.923879504f, -0.382683426f}, {-1.f, -1.22464685e-16f},
+    {-0.923879504f, 0.382683426f}, {-0.707106769f, 0.707106769f}, {-0.382683426f, 0.923879504f},
+    {-1.83697015e-16f, 1.f}, {0.382683426f, 0.923879504f}, {0.707106769f, 0.707106769f},
+    {0.923879504f, 0.382683426f},
 };
 template <int R> struct WOff;
 template <> struct WOff<6> { static constexpr int v = 0; };

@@ -262,10 +262,38 @@ __global__ void __launch_bounds__(256) k_cgemv_n(int M, int K, const cplx<T>* __
   }
 }
 
+// the same with one thread per row i and one sum (GEMM_ONE_SUM), B's few columns broadcast; the K
+// loop is unrolled so that several rows of A are in flight per thread
 template <typename T, int NB>
-static void launch_gemv(int ta, int M, int K, const cplx<T>* A, int64_t lda, const cplx<T>* B, int64_t ldb,
+__global__ void __launch_bounds__(256) k_cgemv_n1(int M, int K, const cplx<T>* __restrict__ A, int64_t lda,
+                                                 const cplx<T>* __restrict__ B, int64_t ldb, Epi<T> epi) {
+  using C = cplx<T>;
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= M) return;
+  C acc[NB];
+#pragma unroll
+  for (int j = 0; j < NB; ++j) acc[j] = czero<C>();
+#pragma unroll 8
+  for (int k = 0; k < K; ++k) {
+    const C x = A[i + (int64_t)k * lda];
+#pragma unroll
+    for (int j = 0; j < NB; ++j) {
+      const C b = B[k + (int64_t)j * ldb];
+      acc[j].x = fma(x.x, b.x, acc[j].x);
+      acc[j].x = fma(-x.y, b.y, acc[j].x);
+      acc[j].y = fma(x.x, b.y, acc[j].y);
+      acc[j].y = fma(x.y, b.x, acc[j].y);
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < NB; ++j) epi_apply<T>(epi, i, j, acc[j]);
+}
+
+template <typename T, int NB>
+static void launch_gemv(int one_sum, int ta, int M, int K, const cplx<T>* A, int64_t lda, const cplx<T>* B, int64_t ldb,
                         const Epi<T>& epi, cudaStream_t st) {
   if (ta == 1) k_cgemv_t<T, NB><<<M, 256, 0, st>>>(M, K, A, lda, B, ldb, epi);
+  else if (one_sum) k_cgemv_n1<T, NB><<<(M + 255) / 256, 256, 0, st>>>(M, K, A, lda, B, ldb, epi);
   else k_cgemv_n<T, NB><<<(M + 63) / 64, 256, 0, st>>>(M, K, A, lda, B, ldb, epi);
   count_launch();
 }
@@ -295,14 +323,16 @@ cudaError_t launch_cgemm(int ta, int tb, int M, int N, int K, const cplx<T>* A, 
                          const cplx<T>* B, int64_t ldb, const Epi<T>& epi, int nsplit, cplx<T>* ws,
                          cudaStream_t st, int tri) {
   if (M <= 0 || N <= 0) return cudaSuccess;
+  const int one_sum = tri & GEMM_ONE_SUM;
+  tri &= ~GEMM_ONE_SUM;
   if (tri == GEMM_LOWER_OUT && M != N) return cudaErrorInvalidValue;
   if (tri == GEMM_B_UPPER && N > K) return cudaErrorInvalidValue;
   if (N <= GEMV_MAXN && tb == 0 && tri == GEMM_FULL && K > 0) {
     switch (N) {
-      case 1: launch_gemv<T, 1>(ta, M, K, A, lda, B, ldb, epi, st); break;
-      case 2: launch_gemv<T, 2>(ta, M, K, A, lda, B, ldb, epi, st); break;
-      case 3: launch_gemv<T, 3>(ta, M, K, A, lda, B, ldb, epi, st); break;
-      default: launch_gemv<T, 4>(ta, M, K, A, lda, B, ldb, epi, st); break;
+      case 1: launch_gemv<T, 1>(one_sum, ta, M, K, A, lda, B, ldb, epi, st); break;
+      case 2: launch_gemv<T, 2>(one_sum, ta, M, K, A, lda, B, ldb, epi, st); break;
+      case 3: launch_gemv<T, 3>(one_sum, ta, M, K, A, lda, B, ldb, epi, st); break;
+      default: launch_gemv<T, 4>(one_sum, ta, M, K, A, lda, B, ldb, epi, st); break;
     }
     return cudaGetLastError();
   }

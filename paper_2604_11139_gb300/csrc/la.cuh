@@ -46,4 +46,10 @@ cudaError_t la_lob_coef(const double2* C, int k, int keep, double2* B, cudaStrea
 template <typename T>
 cudaError_t la_cheb_acc(const cplx<T>* y, int64_t ldy, int npw, int nband, const double* coef, cplx<T>* out,
                         int64_t ldo, int first, cudaStream_t st);
+// the same in the fixed order of operations of the FP64 solve (la_keep.cu)
+cudaError_t la_cholesky_keep(double2* A, int64_t lda, int n, int* flag, cudaStream_t st);
+cudaError_t la_trinv_lower_keep(const double2* L, int64_t lda, int n, double2* X, int64_t ldx, double2* tmp,
+                                cudaStream_t st);
+cudaError_t la_lanczos_keep(const double2* v0, int n, int steps, double2* v, double2* vprev, double2* w, double* ab,
+                            double* bound, ApplyFn apply, void* ctx, cudaStream_t st);
 }  // namespace pw

@@ -250,7 +250,7 @@ Epi<T> epi(int mode, cplx<T>* out, int64_t ldo, T alpha = 1) {
   return e;
 }
 
-// Bands per FFT batch: half-box planes near fft_batch_bytes (complex64 384 MB, complex128 256 MB
+// Bands per FFT batch: half-box planes near fft_batch_bytes (complex64 384 MB, complex128 512 MB
 // unless tuned), a few large launches.
 int band_batch(const pw_ctx* ctx, int nband, size_t elem = 16) {
   const size_t per = (size_t)ctx->sp.nplane * ctx->n[1] * ctx->n[2] * elem;
@@ -409,13 +409,14 @@ int zgemm(pw_ctx* ctx, int ta, int tb, int M, int N, int K, const double2* A, in
   if (M <= 0 || N <= 0) return PW_OK;
   const cudaStream_t st = ctx->stream;
   if (!ctx->fp64_tc || N <= 4 || K <= 0 || !oz::available()) {
-    CU_TRY(launch_cgemm<double>(ta, tb, M, N, K, A, lda, B, ldb, e, dfma_ns, dfma_ws, st, tri), where);
+    CU_TRY(launch_cgemm<double>(ta, tb, M, N, K, A, lda, B, ldb, e, dfma_ns, dfma_ws, st,
+                                tri | (ctx->keep64 ? GEMM_ONE_SUM : 0)), where);
     return PW_OK;
   }
   // Small products: slicing two operands and one chunk of the digit GEMM take 75 us (8 x 16 x 925 as
   // much as 136 x 32 x 14771), the FP64 pipe 29 us for 2^22 complex products over all SMs
   // (the failure-path hook asks for a digit GEMM of any size)
-  if ((double)M * N * K < (double)(1 << 22) && !ctx->test_wait_expiry) {
+  if ((double)M * N * K < (double)(1 << 22) && !ctx->test_wait_expiry && !ctx->keep64) {
     const int tiles = ((M + 15) / 16) * ((N + 15) / 16);
     const int ns = std::max(1, std::min((2 * 152) / tiles, K / 32));
     WS(part, double2, WS_OZPART, (size_t)(ns > 1 ? ns : 0) * M * N + 1);
@@ -921,6 +922,11 @@ int gram_chol(pw_ctx* ctx, const double2* Y, int64_t ldy, const double2* SY, int
               double2* Linv, double2* tmp, int* flag) {
   const cudaStream_t st = ctx->stream;
   PW_TRY(gram_herm(ctx, Y, ldy, SY, lds, m, G));
+  if (ctx->keep64) {
+    CU_TRY(la_cholesky_keep(G, m, m, flag, st), "cholesky");
+    CU_TRY(la_trinv_lower_keep(G, m, m, Linv, m, tmp, st), "triangular inverse");
+    return PW_OK;
+  }
   CU_TRY(la_cholesky(G, m, m, flag, st), "cholesky");
   CU_TRY(la_trinv_lower(G, m, m, Linv, m, tmp, st), "triangular inverse");
   return PW_OK;
@@ -948,7 +954,8 @@ constexpr int kMixedEigMin = 16;
 constexpr int kEigCorrections = 2;
 int eigh_impl(pw_ctx* ctx, double2* A, int n, double2* U, double* eig, double2* jac, double* norms, int* sweeps) {
   const cudaStream_t st = ctx->stream;
-  if (n < kMixedEigMin) return la_jacobi_eigh(A, n, U, eig, jac, norms, st, 40, 1e-13, false, sweeps);
+  const bool keep = ctx->keep64;  // FP32 rotations from n = 128, no corrections, seven digits
+  if (n < (keep ? 128 : kMixedEigMin)) return la_jacobi_eigh(A, n, U, eig, jac, norms, st, 40, 1e-13, false, sweeps);
   const size_t nn = (size_t)n * n;
   const size_t bytes = sizeof(double2) * 5 * nn + sizeof(float2) * (4 * nn + n + 2) + 64;
   WS(mixb, unsigned char, WS_EIGMIX, bytes);
@@ -964,9 +971,9 @@ int eigh_impl(pw_ctx* ctx, double2* A, int n, double2* U, double* eig, double2* 
   // products of n x n matrices: tiles of 16 on the FP64 pipe beat slicing and digits up to 160;
   // eight digits, or the rounding of A' alone (1e-13 of its norm at n = 512) costs another sweep
   auto mul = [&](int ta, int tb, const double2* X, const double2* Y, double2* out, int tri, const char* what) -> int {
-    if (n > 160)
+    if (n > 160 || keep)
       return zgemm(ctx, ta, tb, n, n, n, X, n, Y, n, epi<double>(EPI_STORE, out, n), 1, nullptr, tri, what,
-                   oz::kDigitsFull);
+                   keep ? oz::kDigits : oz::kDigitsFull);
     CU_TRY(launch_cgemm<double>(ta, tb, n, n, n, X, n, Y, n, epi<double>(EPI_STORE, out, n), 1, nullptr, st, tri), what);
     return PW_OK;
   };
@@ -979,19 +986,19 @@ int eigh_impl(pw_ctx* ctx, double2* A, int n, double2* U, double* eig, double2* 
     // Vo = V L^{-dagger}, L L^dagger = V^dagger V
     PW_TRY(mul(1, 0, V, V, Gv, GEMM_FULL, "eig basis Gram"));
     CU_TRY(la_herm_sym(Gv, n, n, st), "eig basis Gram sym");
-    CU_TRY(la_cholesky(Gv, n, n, flag, st), "eig basis Cholesky");
-    CU_TRY(la_trinv_lower(Gv, n, n, Lv, n, T, st), "eig basis triangular inverse");
+    CU_TRY((keep ? la_cholesky_keep : la_cholesky)(Gv, n, n, flag, st), "eig basis Cholesky");
+    CU_TRY((keep ? la_trinv_lower_keep : la_trinv_lower)(Gv, n, n, Lv, n, T, st), "eig basis triangular inverse");
     PW_TRY(mul(0, 1, V, Lv, Vo, GEMM_B_UPPER, "eig basis orthonormalisation"));
     // A' = Vo^dagger A Vo
     PW_TRY(mul(0, 0, A, Vo, T, GEMM_FULL, "eig rotate 1"));
     PW_TRY(mul(1, 0, Vo, T, Gv, GEMM_FULL, "eig rotate 2"));
     CU_TRY(la_herm_sym(Gv, n, n, st), "eig rotated sym");
-    if (it == kEigCorrections) break;
+    if (keep || it == kEigCorrections) break;
     CU_TRY(la_eig_correction(Gv, n, T, st), "eig correction");
     PW_TRY(mul(0, 0, Vo, T, V, GEMM_FULL, "eig corrected basis"));
   }
   PW_TRY(check_flag(ctx, flag, "eigensolver basis Cholesky"));
-  PW_TRY(la_jacobi_eigh(Gv, n, T, eig, jac, norms, st, 40, 1e-13, true, &sw64));
+  PW_TRY(la_jacobi_eigh(Gv, n, T, eig, jac, norms, st, 40, 1e-13, !keep, &sw64));
   PW_TRY(mul(0, 0, Vo, T, U, GEMM_FULL, "eig back-rotation"));
   if (sweeps) *sweeps = sw64;
   return PW_OK;
@@ -1322,7 +1329,11 @@ int bounds_impl(pw_ctx* ctx, const double2* psi, int64_t ld, int nband, int step
     double* ab = (double*)(lz + 3 * npw);
     double* bound = ab + 2 * steps;
     LzCtx lc{ctx};
-    CU_TRY(la_lanczos(v0, npw, steps, lz, lz + npw, lz + 2 * npw, ab, bound, bound + 4, lz_apply, &lc, st), "lanczos");
+    if (ctx->keep64)
+      CU_TRY(la_lanczos_keep(v0, npw, steps, lz, lz + npw, lz + 2 * npw, ab, bound, lz_apply, &lc, st), "lanczos");
+    else
+      CU_TRY(la_lanczos(v0, npw, steps, lz, lz + npw, lz + 2 * npw, ab, bound, bound + 4, lz_apply, &lc, st),
+             "lanczos");
     double h[2];
     CU_TRY(cudaMemcpyAsync(h, bound, 2 * sizeof(double), cudaMemcpyDeviceToHost, st), "bound copy");
     CU_TRY(cudaStreamSynchronize(st), "bound sync");
@@ -1944,6 +1955,12 @@ PW_API int pw_chebfi_solve(pw_ctx* ctx, void* psi_v, int64_t ldpsi, int nband, i
   if (nband == 0) return PW_OK;
   if (!eig) return set_error(PW_EINVAL, "eig is NULL");
   if (precision != PW_FP64 && precision != PW_MIXED) return set_error(PW_EINVAL, "unknown precision");
+  // the FP64 form keeps its order of operations, and with it the phases of its vectors (la_keep.cu)
+  struct Keep {
+    pw_ctx* c;
+    ~Keep() { c->keep64 = false; }
+  } keep{ctx};
+  ctx->keep64 = precision == PW_FP64;
   double2* psi = (double2*)psi_v;
   double rqmin = 0, a = 0, upper = 0;
   if (precision == PW_MIXED) {

@@ -219,7 +219,8 @@ cudaError_t launch_density(const FftPlan& plan, const cplx<T>* tw, const SphereD
 //    and stored (a Hermitian Gram matrix; the tiles above the diagonal are left as they were);
 //  GEMM_B_UPPER: op(B)[k][n] == 0 for k > n (B = L^dagger with L lower triangular), so the K range
 //    of an output tile stops at its last column (N <= K).
-enum { GEMM_FULL = 0, GEMM_LOWER_OUT = 1, GEMM_B_UPPER = 2 };
+//  GEMM_ONE_SUM (a flag beside these): the matrix-vector forms sum over K in one chain per row.
+enum { GEMM_FULL = 0, GEMM_LOWER_OUT = 1, GEMM_B_UPPER = 2, GEMM_ONE_SUM = 4 };
 
 // op(A) is M x K, op(B) is K x N; ta/tb: 0 = as stored (column-major), 1 = conjugate transpose.
 // nsplit > 1 splits K and reduces through `ws` (nsplit*M*N complex) before the epilogue.
@@ -316,8 +317,9 @@ struct pw_ctx {
   uint64_t ws_gen = 0;  // bumped whenever a workspace is (re)allocated (captured graphs check it)
   // tuning: bytes of half-box planes per FFT band batch (complex64, complex128); set by pw_autotune
   // (complex64: large launches beat planes handed over in L2, 10-step filter of 128 bands on
-  // 72 x 72 x 90: 5.6 ms at 48 MB, 4.8 at 384 MB)
-  size_t fft_batch_bytes[2] = {(size_t)384 << 20, (size_t)256 << 20};
+  // 72 x 72 x 90: 5.6 ms at 48 MB, 4.8 at 384 MB; complex128 the same, density of 256 bands on 96^3:
+  // 5.53 ms at 256 MB, 5.30 at 512 MB, the FP64 filter there 103.5 and 102.2 ms)
+  size_t fft_batch_bytes[2] = {(size_t)384 << 20, (size_t)512 << 20};
   // FFT pass kernel forms per precision, variant = xline form + 8 * plane form.  x-line
   // forms: 0 line groups of 1-8 threads with shared-memory twiddles, 1 one thread per line
   // with compile-time twiddles, 2 groups of warps per 32 lines (lane = line) with
@@ -331,6 +333,7 @@ struct pw_ctx {
   // column-slice plane kernels (plane form 3), which fall back to line groups where they do
   // not apply (1.2x the line-group form on the 120^3 box)
   int fft_variant[2] = {8 + 3 * pw::kFormStride, 3 * pw::kFormStride};
+  bool keep64 = false;  // inside an FP64 pw_chebfi_solve: fixed order of operations (la_keep.cu)
   int last_sweeps = 0;  // Jacobi sweeps of the last Rayleigh-Ritz step
   // K splits of the mixed projection GEMM per column count, chosen by pw_autotune (columns ->
   // splits); other column counts use the whole-waves rule
