@@ -139,7 +139,8 @@ __global__ void __launch_bounds__(kThreads) k_fl_zinv(const C* __restrict__ psi,
   }
 }
 
-template <bool REC>
+// REC: 0 the kinetic term, 1 the recurrence, 2 the recurrence without P Z
+template <int REC>
 __global__ void __launch_bounds__(kThreads) k_fl_zfwd(const C* __restrict__ hb, int64_t hb_bs, SphereDev sp, Dim d,
                                                       int n2, const float* __restrict__ kin,
                                                       const C* __restrict__ psi, int64_t ldpsi, C* __restrict__ out,
@@ -197,7 +198,7 @@ __global__ void __launch_bounds__(kThreads) k_fl_zfwd(const C* __restrict__ hb, 
       if constexpr (!REC) {
         o[gg] = make_float2(k * yy.x + v.x, k * yy.y + v.y);
       } else {
-        const C pz = rec.pz ? rec.pz[(int64_t)b * rec.ldpz + gg] : make_float2(0.f, 0.f);
+        const C pz = REC == 1 ? rec.pz[(int64_t)b * rec.ldpz + gg] : make_float2(0.f, 0.f);
         C t = make_float2(ra * (k * yy.x + v.x + pz.x - rs * yy.x), ra * (k * yy.y + v.y + pz.y - rs * yy.y));
         if (rec.ykm1) {
           const C ym = rec.ykm1[(int64_t)b * rec.ldykm1 + gg];
@@ -401,14 +402,17 @@ cudaError_t forward_planes(const FftPlan& plan, const C* tw, const SphereDev& sp
   const int nc = (dz.n + 31) / 32;
   const size_t smz = line_bytes(dz), smy = line_bytes(dy) + sizeof(int) * dy.n;
   cudaError_t e;
-  if ((e = smem_attr(k_fl_yfwd, smy)) || (e = smem_attr(k_fl_zfwd<false>, smz)) || (e = smem_attr(k_fl_zfwd<true>, smz)))
+  if ((e = smem_attr(k_fl_yfwd, smy)) || (e = smem_attr(k_fl_zfwd<0>, smz)) || (e = smem_attr(k_fl_zfwd<1>, smz)) ||
+      (e = smem_attr(k_fl_zfwd<2>, smz)))
     return e;
   k_fl_yfwd<<<dim3(sp.nplane * nc, nb), kThreads, smy, st>>>(hb, hb_bs, sp, dy, dz.n, nc); count_launch();
   const dim3 g((sp.nrow + 31) / 32, nb);
-  if (rec)
-    k_fl_zfwd<true><<<g, kThreads, smz, st>>>(hb, hb_bs, sp, dz, dy.n, kin, psi, ldpsi, out, ldout, *rec);
+  if (rec && !rec->pz)
+    k_fl_zfwd<2><<<g, kThreads, smz, st>>>(hb, hb_bs, sp, dz, dy.n, kin, psi, ldpsi, out, ldout, *rec);
+  else if (rec)
+    k_fl_zfwd<1><<<g, kThreads, smz, st>>>(hb, hb_bs, sp, dz, dy.n, kin, psi, ldpsi, out, ldout, *rec);
   else
-    k_fl_zfwd<false><<<g, kThreads, smz, st>>>(hb, hb_bs, sp, dz, dy.n, kin, psi, ldpsi, out, ldout, Pass3Rec{});
+    k_fl_zfwd<0><<<g, kThreads, smz, st>>>(hb, hb_bs, sp, dz, dy.n, kin, psi, ldpsi, out, ldout, Pass3Rec{});
   count_launch();
   return cudaGetLastError();
 }

@@ -2036,7 +2036,7 @@ __global__ void __launch_bounds__(PlaneW<N2, N3, TW>::THREADS) k_plane_inv_wgp(c
 // receive the plane's blocks of Y_k and t_G by asynchronous copies that the caller issued
 // (committed as the group before any it issues in `before_gather`); `before_gather` runs
 // after the z-lines and waits for them.
-template <typename T, int N2, int N3, int TW, bool REC, typename G>
+template <typename T, int N2, int N3, int TW, int REC, typename G>
 __device__ __forceinline__ void plane_fwd_wg_item(int p, int b, const cplx<T>* __restrict__ hb, int64_t hb_bs,
                                                   const SphereDev& sp, const FftPlan& plan,
                                                   const cplx<T>* __restrict__ tw, const cplx<T>* __restrict__ psi,
@@ -2155,7 +2155,7 @@ __device__ __forceinline__ void plane_fwd_wg_item(int p, int b, const cplx<T>* _
       if constexpr (!REC) {
         o[gg] = mk<C>(k * yy.x + v.x, k * yy.y + v.y);
       } else {
-        const C pz = rec.pz ? ((const C*)rec.pz)[(int64_t)b * rec.ldpz + gg] : czero<C>();
+        const C pz = REC == 1 ? ((const C*)rec.pz)[(int64_t)b * rec.ldpz + gg] : czero<C>();
         C r = mk<C>(ra * (k * yy.x + v.x + pz.x - rs * yy.x), ra * (k * yy.y + v.y + pz.y - rs * yy.y));
         if (rec.ykm1) {
           const C ym = ((const C*)rec.ykm1)[(int64_t)b * rec.ldykm1 + gg];
@@ -2198,7 +2198,7 @@ __device__ __forceinline__ void plane_fwd_stage(const SphereDev& sp, int p, int 
 
 // one CTA per (plane, band): the plane's blocks of Y_k and t_G are copied while the y- and
 // z-lines are transformed
-template <typename T, int N2, int N3, int TW, bool REC>
+template <typename T, int N2, int N3, int TW, int REC>
 __global__ void __launch_bounds__(PlaneW<N2, N3, TW>::THREADS) k_plane_fwd_wg(const cplx<T>* __restrict__ hb,
                                                                                int64_t hb_bs, SphereDev sp, FftPlan plan,
                                                                                const cplx<T>* __restrict__ tw,
@@ -2219,7 +2219,7 @@ __global__ void __launch_bounds__(PlaneW<N2, N3, TW>::THREADS) k_plane_fwd_wg(co
 // Persistent form: one CTA per SM walks the (plane, band) items; while an item's coefficients
 // are gathered, the next item's half-box plane is prefetched into L2 (one bulk prefetch of the
 // contiguous plane) and its blocks of Y_k and t_G are copied into the other of two buffers.
-template <typename T, int N2, int N3, int TW, bool REC>
+template <typename T, int N2, int N3, int TW, int REC>
 __global__ void __launch_bounds__(PlaneW<N2, N3, TW>::THREADS) k_plane_fwd_wgp(const cplx<T>* __restrict__ hb,
                                                                                 int64_t hb_bs, SphereDev sp,
                                                                                 FftPlan plan,
@@ -2293,22 +2293,28 @@ static cudaError_t plane_wg_pair(int which, const cplx<T>* psi, int64_t ldpsi, c
       };
       if (rec) {
         if constexpr (std::is_same<T, float>::value) {
-          if ((e = cudaFuncSetAttribute(k_plane_fwd_wgp<T, N2, N3, TW, true>,
+          auto run = [&](auto rc) -> cudaError_t {  // 1 with P Z, 2 without
+            constexpr int R = decltype(rc)::value;
+          if ((e = cudaFuncSetAttribute(k_plane_fwd_wgp<T, N2, N3, TW, R>,
                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)))
             return e;
-          const int grid = grid_of((const void*)k_plane_fwd_wgp<T, N2, N3, TW, true>);
-          k_plane_fwd_wgp<T, N2, N3, TW, true><<<grid, PW::THREADS, sm, st>>>(hb, hb_bs, sp, plan, tw, kin, psi,
+          const int grid = grid_of((const void*)k_plane_fwd_wgp<T, N2, N3, TW, R>);
+          k_plane_fwd_wgp<T, N2, N3, TW, R><<<grid, PW::THREADS, sm, st>>>(hb, hb_bs, sp, plan, tw, kin, psi,
                                                                              ldpsi, out, ldout, *rec, nb);
           count_launch();
+            return cudaSuccess;
+          };
+          e = rec->pz ? run(std::integral_constant<int, 1>{}) : run(std::integral_constant<int, 2>{});
+          if (e) return e;
         } else {
           return cudaErrorNotSupported;
         }
       } else {
-        if ((e = cudaFuncSetAttribute(k_plane_fwd_wgp<T, N2, N3, TW, false>,
+        if ((e = cudaFuncSetAttribute(k_plane_fwd_wgp<T, N2, N3, TW, 0>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)))
           return e;
         const int grid = grid_of((const void*)k_plane_fwd_wgp<T, N2, N3, TW, false>);
-        k_plane_fwd_wgp<T, N2, N3, TW, false><<<grid, PW::THREADS, sm, st>>>(hb, hb_bs, sp, plan, tw, kin, psi,
+        k_plane_fwd_wgp<T, N2, N3, TW, 0><<<grid, PW::THREADS, sm, st>>>(hb, hb_bs, sp, plan, tw, kin, psi,
                                                                             ldpsi, out, ldout, Pass3Rec{}, nb);
         count_launch();
       }
@@ -2340,25 +2346,31 @@ static cudaError_t plane_wg_pair(int which, const cplx<T>* psi, int64_t ldpsi, c
     } else {
       if (rec) {
         if constexpr (std::is_same<T, float>::value) {
-          if ((e = cudaFuncSetAttribute(k_plane_fwd_wg<T, N2, N3, TW, true>,
+          auto run = [&](auto rc) -> cudaError_t {  // 1 with P Z, 2 without
+            constexpr int R = decltype(rc)::value;
+          if ((e = cudaFuncSetAttribute(k_plane_fwd_wg<T, N2, N3, TW, R>,
                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)))
             return e;
-          if ((e = cudaFuncSetAttribute(k_plane_fwd_wg<T, N2, N3, TW, true>,
+          if ((e = cudaFuncSetAttribute(k_plane_fwd_wg<T, N2, N3, TW, R>,
                                         cudaFuncAttributePreferredSharedMemoryCarveout, 100)))
             return e;
-          k_plane_fwd_wg<T, N2, N3, TW, true><<<dim3(sp.nplane, nb), PW::THREADS, sm, st>>>(
+          k_plane_fwd_wg<T, N2, N3, TW, R><<<dim3(sp.nplane, nb), PW::THREADS, sm, st>>>(
               hb, hb_bs, sp, plan, tw, kin, psi, ldpsi, out, ldout, *rec); count_launch();
+            return cudaSuccess;
+          };
+          e = rec->pz ? run(std::integral_constant<int, 1>{}) : run(std::integral_constant<int, 2>{});
+          if (e) return e;
         } else {
           return cudaErrorNotSupported;
         }
       } else {
-        if ((e = cudaFuncSetAttribute(k_plane_fwd_wg<T, N2, N3, TW, false>,
+        if ((e = cudaFuncSetAttribute(k_plane_fwd_wg<T, N2, N3, TW, 0>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)))
           return e;
-        if ((e = cudaFuncSetAttribute(k_plane_fwd_wg<T, N2, N3, TW, false>,
+        if ((e = cudaFuncSetAttribute(k_plane_fwd_wg<T, N2, N3, TW, 0>,
                                       cudaFuncAttributePreferredSharedMemoryCarveout, 100)))
           return e;
-        k_plane_fwd_wg<T, N2, N3, TW, false><<<dim3(sp.nplane, nb), PW::THREADS, sm, st>>>(
+        k_plane_fwd_wg<T, N2, N3, TW, 0><<<dim3(sp.nplane, nb), PW::THREADS, sm, st>>>(
             hb, hb_bs, sp, plan, tw, kin, psi, ldpsi, out, ldout, Pass3Rec{}); count_launch();
       }
     }
@@ -2501,7 +2513,7 @@ __global__ void __launch_bounds__(PlaneR<N2, N3, TW>::THREADS) k_plane_inv_rs(co
   }
 }
 
-template <typename T, int N2, int N3, int TW, bool REC>
+template <typename T, int N2, int N3, int TW, int REC>
 __global__ void __launch_bounds__(PlaneR<N2, N3, TW>::THREADS) k_plane_fwd_rs(const cplx<T>* __restrict__ hb,
                                                                                int64_t hb_bs, SphereDev sp, FftPlan plan,
                                                                                const cplx<T>* __restrict__ tw,
@@ -2622,7 +2634,7 @@ __global__ void __launch_bounds__(PlaneR<N2, N3, TW>::THREADS) k_plane_fwd_rs(co
       if constexpr (!REC) {
         o[gg] = mk<C>(k * yy.x + v.x, k * yy.y + v.y);
       } else {
-        const C pz = rec.pz ? ((const C*)rec.pz)[(int64_t)b * rec.ldpz + gg] : czero<C>();
+        const C pz = REC == 1 ? ((const C*)rec.pz)[(int64_t)b * rec.ldpz + gg] : czero<C>();
         C r = mk<C>(ra * (k * yy.x + v.x + pz.x - rs * yy.x), ra * (k * yy.y + v.y + pz.y - rs * yy.y));
         if (rec.ykm1) {
           const C ym = ((const C*)rec.ykm1)[(int64_t)b * rec.ldykm1 + gg];
@@ -2676,17 +2688,23 @@ static cudaError_t plane_rs_pair(int which, const cplx<T>* psi, int64_t ldpsi, c
       k_plane_inv_rs<T, N2, N3, TW><<<grid, PR::THREADS, sm, st>>>(psi, ldpsi, hb, hb_bs, sp, plan, tw); count_launch();
     } else if (rec) {
       if constexpr (kF32) {
-        if ((e = cudaFuncSetAttribute(k_plane_fwd_rs<T, N2, N3, TW, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+          auto run = [&](auto rc) -> cudaError_t {  // 1 with P Z, 2 without
+            constexpr int R = decltype(rc)::value;
+        if ((e = cudaFuncSetAttribute(k_plane_fwd_rs<T, N2, N3, TW, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)sm)))
           return e;
-        k_plane_fwd_rs<T, N2, N3, TW, true><<<grid, PR::THREADS, sm, st>>>(hb, hb_bs, sp, plan, tw, kin, psi, ldpsi,
+        k_plane_fwd_rs<T, N2, N3, TW, R><<<grid, PR::THREADS, sm, st>>>(hb, hb_bs, sp, plan, tw, kin, psi, ldpsi,
                                                                           out, ldout, *rec); count_launch();
-      }
+            return cudaSuccess;
+          };
+          e = rec->pz ? run(std::integral_constant<int, 1>{}) : run(std::integral_constant<int, 2>{});
+          if (e) return e;
+        }
     } else {
-      if ((e = cudaFuncSetAttribute(k_plane_fwd_rs<T, N2, N3, TW, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      if ((e = cudaFuncSetAttribute(k_plane_fwd_rs<T, N2, N3, TW, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)sm)))
         return e;
-      k_plane_fwd_rs<T, N2, N3, TW, false><<<grid, PR::THREADS, sm, st>>>(hb, hb_bs, sp, plan, tw, kin, psi, ldpsi,
+      k_plane_fwd_rs<T, N2, N3, TW, 0><<<grid, PR::THREADS, sm, st>>>(hb, hb_bs, sp, plan, tw, kin, psi, ldpsi,
                                                                          out, ldout, Pass3Rec{}); count_launch();
     }
     return cudaGetLastError();
