@@ -110,6 +110,10 @@ __device__ __forceinline__ ll mulv(int al, int ah, int vl, int vh) {
   return madw(ah, vh, sext_hi(m));
 }
 
+// the shift that brings the larger component of v (|v| <= 2^62.4) to 2^61 .. 2^62
+__device__ __forceinline__ int up_shift(fc v) {
+  return max(__clzll((v.x ^ (v.x >> 63)) | (v.y ^ (v.y >> 63))) - 2, 0);
+}
 // round(Re(conj(a) b) / 2^64)
 __device__ __forceinline__ ll dot64(fc a, fc b) {
   const int axl = lo32(a.x), axh = hi32(a.x), ayl = lo32(a.y), ayh = hi32(a.y);
@@ -702,22 +706,22 @@ __global__ void __launch_bounds__(kThreads, BIG ? 2 : 3) k_fx_x(double2* __restr
 
 // ---- density: inverse x of a (and b), out[r] += sum_b w_b Re[conj(a) b] --------------------------
 // 32 lines per CTA and a share of the bands (blockIdx.y); the sums stay in shared memory until the
-// end and are added to the permuted grid atomically.  The products are integers too, of the values
-// shifted up to 2^62 by what the line's 2-norm allows (|value| <= sqrt(np) times it): one conversion
-// and one FMA per point are left to the FP64 pipe, which was the bound with FP64 products.
+// end and are added to the permuted grid atomically.  The products are integers too: one conversion
+// and one FMA per point are left to the FP64 pipe, which was the bound with FP64 products.  Each
+// value is shifted up to 2^62 by its own leading zeros first, so that a product keeps 2^-58 of
+// itself: where a band has died away the density is as close as the transform left the band, not
+// one unit of the line's largest product.
 template <bool BIG>
 __global__ void __launch_bounds__(kThreads, BIG ? 2 : 3) k_fx_dens(const double2* __restrict__ hba,
                                                          const double2* __restrict__ hbb, int64_t hb_bs, int nb,
                                                          int bper, const double* __restrict__ wgt, int np, int nyz,
-                                                         Dim d, int bits, int room,
-                                                         double* __restrict__ out_perm) {
+                                                         Dim d, int bits, double* __restrict__ out_perm) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, n = d.n;
   fc* bufa = reinterpret_cast<fc*>(smem);
   fc* bufb = bufa + (hbb ? n * PT : 0);
   double* acc = reinterpret_cast<double*>(bufb + n * PT) + lane;  // [n][32]
   __shared__ unsigned red[2][kWarps][32];
-  __shared__ ll red2[2][kWarps][32];
   const int yz = blockIdx.x * 32 + lane;
   const bool live = yz < nyz;
   for (int e = w; e < n; e += kWarps) acc[e * 32] = 0.0;
@@ -740,25 +744,17 @@ __global__ void __launch_bounds__(kThreads, BIG ? 2 : 3) k_fx_dens(const double2
       const int E = top_exp(mx);
       const In in(E, bits);
       (which ? kb : ka) = out_exp(mx, E - bits + 2);
-      ll ss = 0;
 #define FX_F(R)                                              \
   _Pragma("unroll 1") for (int J = w; J < d.r2; J += kWarps) \
-      inv1<R, true>(col, J, d, in, [&](int e) { return e < np; }, &ss)
+      inv1<R>(col, J, d, in, [&](int e) { return e < np; })
       FX_SWITCH(d.r1, FX_F)
 #undef FX_F
-      red2[which][w][lane] = ss;
     }
     __syncthreads();
-    auto shift = [&](int which) {
-      ll ss = 1;
-#pragma unroll
-      for (int i = 0; i < kWarps; ++i) ss += red2[which][i][lane];
-      return min(max((__clzll(ss) - room) >> 1, 0), 12);
-    };
-    const int ta = shift(0), tb = hbb ? shift(1) : ta;
     if (!hbb) kb = ka;
-    const Out of{ka == kNan || kb == kNan ? kNan : ka + kb - ta - tb + 64};
-    const double wb = wgt[b];
+    const bool bad = ka == kNan || kb == kNan;
+    const int kab = bad ? 0 : ka + kb + 64;
+    const double wb = bad ? __longlong_as_double(0x7ff8000000000000ll) : wgt[b];
     // the last stage of a (and b); with b, a's values go back to its line
 #define FX_F(R)                                                                   \
   _Pragma("unroll 1") for (int blk = w; blk < d.r1; blk += kWarps) {              \
@@ -767,16 +763,23 @@ __global__ void __launch_bounds__(kThreads, BIG ? 2 : 3) k_fx_dens(const double2
       fc* ca = bufa + lane + blk * R * PT;                                        \
       _Pragma("unroll") for (int m = 0; m < R; ++m) y[m] = ca[m * PT];            \
       dft<+1, R>(y);                                                              \
-      _Pragma("unroll") for (int m = 0; m < R; ++m) ca[m * PT] = {y[m].x << ta, y[m].y << ta}; \
+      _Pragma("unroll") for (int m = 0; m < R; ++m) ca[m * PT] = y[m];                  \
     }                                                                             \
     const fc* cb = bufb + lane + blk * R * PT;                                    \
     _Pragma("unroll") for (int m = 0; m < R; ++m) y[m] = cb[m * PT];              \
     dft<+1, R>(y);                                                                \
     _Pragma("unroll") for (int m = 0; m < R; ++m) {                               \
+      const int tb = up_shift(y[m]);                                              \
       const fc vb = {y[m].x << tb, y[m].y << tb};                                 \
-      const fc va = hbb ? bufa[lane + (blk * R + m) * PT] : vb;                   \
+      int ta = tb;                                                                \
+      fc va = vb;                                                                 \
+      if (hbb) {                                                                  \
+        va = bufa[lane + (blk * R + m) * PT];                                     \
+        ta = up_shift(va);                                                        \
+        va = {va.x << ta, va.y << ta};                                            \
+      }                                                                           \
       double* s = &acc[(blk * R + m) * 32];                                       \
-      *s = fma(wb, of(dot64(va, vb)), *s);                                        \
+      *s = fma(wb, Out{kab - ta - tb}(dot64(va, vb)), *s);                        \
     }                                                                             \
   }
     FX_SWITCH(d.r2, FX_F)
@@ -914,11 +917,6 @@ cudaError_t local_apply(const FftPlan& plan, const double2* tw, const SphereDev&
   return cudaGetLastError();
 }
 
-// The same for the density: the values, at most sqrt(np) 2^(x - 2 + t), stay below 2^62.
-static int room_dens(int np) {
-  return (int)ceil(64.0 - 2.0 * (62.0 + 2.0 - 0.5 * log2((double)np) - 32.0));
-}
-
 cudaError_t density(const FftPlan& plan, const double2* tw, const SphereDev& sp, const double2* a, const double2* b,
                     int64_t ld, int nband, const double* w_dev, double* out_perm, double2* hb, int band_batch,
                     cudaStream_t st) {
@@ -929,7 +927,7 @@ cudaError_t density(const FftPlan& plan, const double2* tw, const SphereDev& sp,
   const size_t line = sizeof(fc) * PT;
   const size_t smz = line * dz.n, smy = line * dy.n + sizeof(int) * dy.n;
   const size_t smx = line * dx.n * (b ? 2 : 1) + sizeof(double) * 32 * dx.n;
-  if (smx > 220 * 1024) return cudaErrorNotSupported;  // 6 KB more are static
+  if (smx > 220 * 1024) return cudaErrorNotSupported;  // 2 KB more are static
   cudaError_t e;
   auto attr = [&](const void* f, size_t sm) {
     return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
@@ -950,8 +948,7 @@ cudaError_t density(const FftPlan& plan, const double2* tw, const SphereDev& sp,
     int splits = std::max(1, std::min(nb, (152 * 4 + gx - 1) / gx));
     const int bper = (nb + splits - 1) / splits;
     splits = (nb + bper - 1) / bper;
-    (big(dx) ? k_fx_dens<true> : k_fx_dens<false>)<<<dim3(gx, splits), kThreads, smx, st>>>(hb, hbb, hb_bs, nb, bper, w_dev + b0, sp.nplane, nyz, dx, bx,
-                                                       room_dens(sp.nplane), out_perm); count_launch();
+    (big(dx) ? k_fx_dens<true> : k_fx_dens<false>)<<<dim3(gx, splits), kThreads, smx, st>>>(hb, hbb, hb_bs, nb, bper, w_dev + b0, sp.nplane, nyz, dx, bx, out_perm); count_launch();
   }
   return cudaGetLastError();
 }
