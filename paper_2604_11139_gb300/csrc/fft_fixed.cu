@@ -263,9 +263,8 @@ __device__ __forceinline__ unsigned track(unsigned m, double2 v) {
   m = max(m, (unsigned)__double2hiint(v.x) & 0x7fffffffu);
   return max(m, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
 }
-// E with every |component| < 2^E, from the largest high word; values below 2^-900 count as that
-// small, which keeps the scales normal numbers
-__device__ __forceinline__ int top_exp(unsigned m) { return max((int)(m >> 20) - 1022, -900); }
+// E with every |component| < 2^E, from the largest high word (subnormal values count as zero)
+__device__ __forceinline__ int top_exp(unsigned m) { return (int)(m >> 20) - 1022; }
 constexpr int kNan = 1 << 30;  // Out::k of a line with a component that is not finite
 
 // FP64 -> round(x 2^(bits - E)): the power of two goes into the exponent field by an integer
@@ -292,8 +291,8 @@ struct Out {
     const int hi = __double2hiint(d);
     if ((unsigned)(k + 900) <= 1800u) return __hiloint2double(hi ? hi + k * (1 << 20) : 0, __double2loint(d));
     if (k == kNan) return __longlong_as_double(0x7ff8000000000000ll);
-    const int h = k / 2;
-    return d * __hiloint2double((h + 1023) << 20, 0) * __hiloint2double((k - h + 1023) << 20, 0);
+    const int kc = max(k, -2040), h = kc / 2;  // 2^63 2^-2040 is 0 already
+    return d * __hiloint2double((h + 1023) << 20, 0) * __hiloint2double((kc - h + 1023) << 20, 0);
   }
   __device__ __forceinline__ double2 operator()(fc v) const { return make_double2((*this)(v.x), (*this)(v.y)); }
 };
