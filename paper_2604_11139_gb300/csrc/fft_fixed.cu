@@ -299,6 +299,7 @@ struct Out {
 __device__ __forceinline__ int out_exp(unsigned m, int k) { return m >= 0x7ff00000u ? kNan : k; }
 
 constexpr int kWarps = 8, kThreads = 32 * kWarps;
+constexpr int kDynSmem = 224 * 1024;  // limit of dynamic shared memory; up to 3 KB are static
 constexpr int PT = 33;  // pitch of an element's 32 lines: lane-wise and line-wise accesses are conflict-free
 
 struct Dim {
@@ -886,12 +887,9 @@ cudaError_t local_apply(const FftPlan& plan, const double2* tw, const SphereDev&
   const size_t line = sizeof(fc) * PT;
   const size_t smz = line * dz.n, smy = line * dy.n + sizeof(int) * dy.n, smx = line * dx.n;
   cudaError_t e;
-  auto attr = [&](const void* f, size_t sm) {
-    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  };
-  if ((e = attr(big(dz) ? (const void*)k_fx_zinv<true> : (const void*)k_fx_zinv<false>, smz)) || (e = attr(big(dz) ? (const void*)k_fx_zfwd<true> : (const void*)k_fx_zfwd<false>, smz)) ||
-      (e = attr(big(dy) ? (const void*)k_fx_yinv<true> : (const void*)k_fx_yinv<false>, smy)) || (e = attr(big(dy) ? (const void*)k_fx_yfwd<true> : (const void*)k_fx_yfwd<false>, smy)) ||
-      (e = attr(big(dx) ? (const void*)k_fx_x<true> : (const void*)k_fx_x<false>, smx)))
+  if ((e = smem_limit(big(dz) ? k_fx_zinv<true> : k_fx_zinv<false>, smz, kDynSmem)) || (e = smem_limit(big(dz) ? k_fx_zfwd<true> : k_fx_zfwd<false>, smz, kDynSmem)) ||
+      (e = smem_limit(big(dy) ? k_fx_yinv<true> : k_fx_yinv<false>, smy, kDynSmem)) || (e = smem_limit(big(dy) ? k_fx_yfwd<true> : k_fx_yfwd<false>, smy, kDynSmem)) ||
+      (e = smem_limit(big(dx) ? k_fx_x<true> : k_fx_x<false>, smx, kDynSmem)))
     return e;
   const int bz = bits_line(dz), by = bits_line(dy), bx = bits_x(dx, sp.nplane), rx = room_x(dx, sp.nplane);
   for (int b0 = 0; b0 < nband; b0 += band_batch) {
@@ -926,13 +924,10 @@ cudaError_t density(const FftPlan& plan, const double2* tw, const SphereDev& sp,
   const size_t line = sizeof(fc) * PT;
   const size_t smz = line * dz.n, smy = line * dy.n + sizeof(int) * dy.n;
   const size_t smx = line * dx.n * (b ? 2 : 1) + sizeof(double) * 32 * dx.n;
-  if (smx > 220 * 1024) return cudaErrorNotSupported;  // 2 KB more are static
+  if (smx > 220 * 1024) return cudaErrorNotSupported;
   cudaError_t e;
-  auto attr = [&](const void* f, size_t sm) {
-    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  };
-  if ((e = attr(big(dz) ? (const void*)k_fx_zinv<true> : (const void*)k_fx_zinv<false>, smz)) || (e = attr(big(dy) ? (const void*)k_fx_yinv<true> : (const void*)k_fx_yinv<false>, smy)) ||
-      (e = attr(big(dx) ? (const void*)k_fx_dens<true> : (const void*)k_fx_dens<false>, smx)))
+  if ((e = smem_limit(big(dz) ? k_fx_zinv<true> : k_fx_zinv<false>, smz, kDynSmem)) || (e = smem_limit(big(dy) ? k_fx_yinv<true> : k_fx_yinv<false>, smy, kDynSmem)) ||
+      (e = smem_limit(big(dx) ? k_fx_dens<true> : k_fx_dens<false>, smx, kDynSmem)))
     return e;
   const int bz = bits_line(dz), by = bits_line(dy), bx = bits_line(dx);
   double2* hbb = b ? hb + hb_bs * band_batch : nullptr;

@@ -368,9 +368,6 @@ static Dim dim_of(const FftPlan& plan, const C* tw, int i) {
   return {f.n, f.radix[0], f.radix[1], tw + f.tw_off[0]};
 }
 static size_t line_bytes(const Dim& d) { return sizeof(C) * PT * d.n; }
-template <typename F> static cudaError_t smem_attr(F* f, size_t sm) {
-  return cudaFuncSetAttribute((const void*)f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-}
 
 cudaError_t inverse_planes(const FftPlan& plan, const C* tw, const SphereDev& sp, const C* psi, int64_t ldpsi, C* hb,
                            int64_t hb_bs, int nb, cudaStream_t st) {
@@ -378,7 +375,7 @@ cudaError_t inverse_planes(const FftPlan& plan, const C* tw, const SphereDev& sp
   const int nc = (dz.n + 31) / 32;
   const size_t smz = line_bytes(dz), smy = line_bytes(dy) + sizeof(int) * dy.n;
   cudaError_t e;
-  if ((e = smem_attr(k_fl_zinv, smz)) || (e = smem_attr(k_fl_yinv, smy))) return e;
+  if ((e = smem_limit(k_fl_zinv, smz)) || (e = smem_limit(k_fl_yinv, smy))) return e;
   k_fl_zinv<<<dim3((sp.nrow + 31) / 32, nb), kThreads, smz, st>>>(psi, ldpsi, hb, hb_bs, sp, dz, dy.n); count_launch();
   k_fl_yinv<<<dim3(sp.nplane * nc, nb), kThreads, smy, st>>>(hb, hb_bs, sp, dy, dz.n, nc); count_launch();
   return cudaGetLastError();
@@ -390,7 +387,7 @@ cudaError_t xlines(const FftPlan& plan, const C* tw, const SphereDev& sp, const 
   const int nyz = plan.n[1] * plan.n[2];
   const size_t sm = line_bytes(dx);
   cudaError_t e;
-  if ((e = smem_attr(k_fl_x, sm))) return e;
+  if ((e = smem_limit(k_fl_x, sm))) return e;
   k_fl_x<<<dim3((nyz + 31) / 32, nb), kThreads, sm, st>>>(hb, hb_bs, vperm, sp.nplane, nyz, dx); count_launch();
   return cudaGetLastError();
 }
@@ -402,8 +399,8 @@ cudaError_t forward_planes(const FftPlan& plan, const C* tw, const SphereDev& sp
   const int nc = (dz.n + 31) / 32;
   const size_t smz = line_bytes(dz), smy = line_bytes(dy) + sizeof(int) * dy.n;
   cudaError_t e;
-  if ((e = smem_attr(k_fl_yfwd, smy)) || (e = smem_attr(k_fl_zfwd<0>, smz)) || (e = smem_attr(k_fl_zfwd<1>, smz)) ||
-      (e = smem_attr(k_fl_zfwd<2>, smz)))
+  if ((e = smem_limit(k_fl_yfwd, smy)) || (e = smem_limit(k_fl_zfwd<0>, smz)) || (e = smem_limit(k_fl_zfwd<1>, smz)) ||
+      (e = smem_limit(k_fl_zfwd<2>, smz)))
     return e;
   k_fl_yfwd<<<dim3(sp.nplane * nc, nb), kThreads, smy, st>>>(hb, hb_bs, sp, dy, dz.n, nc); count_launch();
   const dim3 g((sp.nrow + 31) / 32, nb);

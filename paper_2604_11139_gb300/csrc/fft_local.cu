@@ -415,7 +415,7 @@ static cudaError_t launch_xline_fused(cplx<T>* hb, int64_t hb_bs, const T* vperm
                                       const FftPlan& plan, const cplx<T>* tw, int nb, cudaStream_t st) {
   using LC = LineCfg<N1>;
   const size_t sm = sizeof(cplx<T>) * ((size_t)LC::LPC * LC::NP + plan.d[0].tw_count);
-  cudaError_t e = cudaFuncSetAttribute(k_xline_fused<T, N1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  cudaError_t e = smem_limit(k_xline_fused<T, N1>, sm);
   if (e) return e;
   const int nyz = plan.n[1] * plan.n[2];
   k_xline_fused<T, N1><<<dim3((nyz + LC::LPC - 1) / LC::LPC, nb), LC::THREADS, sm, st>>>(hb, hb_bs, vperm, sp, plan, tw); count_launch();
@@ -427,7 +427,7 @@ static cudaError_t launch_xline_lg(cplx<T>* hb, int64_t hb_bs, const T* vperm, c
                                    const FftPlan& plan, const cplx<T>* tw, int nb, cudaStream_t st) {
   using LC = LineCfg<N1>;
   const size_t sm = sizeof(cplx<T>) * ((size_t)LC::LPC * LC::NP + plan.d[0].tw_count);
-  cudaError_t e = cudaFuncSetAttribute(k_xline_lg<T, N1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  cudaError_t e = smem_limit(k_xline_lg<T, N1>, sm);
   if (e) return e;
   const int nyz = plan.n[1] * plan.n[2];
   k_xline_lg<T, N1><<<dim3((nyz + LC::LPC - 1) / LC::LPC, nb), LC::THREADS, sm, st>>>(hb, hb_bs, vperm, sp, plan, tw); count_launch();
@@ -1001,13 +1001,11 @@ static cudaError_t plane_lg_pair(int which, const cplx<T>* psi, int64_t ldpsi, c
     const size_t smf = plane_f_smem<T, N2, N3>(sp, plan);
     if (smf <= 227 * 1024) {
       if (which == 0) {
-        if ((e = cudaFuncSetAttribute(k_plane_inv_f<T, N2, N3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smf)))
+        if ((e = smem_limit(k_plane_inv_f<T, N2, N3>, smf)))
           return e;
         k_plane_inv_f<T, N2, N3><<<dim3(sp.nplane, nb), 256, smf, st>>>(psi, ldpsi, hb, hb_bs, sp, plan, tw); count_launch();
       } else {
-        if ((e = cudaFuncSetAttribute(k_plane_fwd_f<T, N2, N3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smf)))
+        if ((e = smem_limit(k_plane_fwd_f<T, N2, N3>, smf)))
           return e;
         k_plane_fwd_f<T, N2, N3><<<dim3(sp.nplane, nb), 256, smf, st>>>(hb, hb_bs, sp, plan, tw, kin, psi, ldpsi, out,
                                                                        ldout); count_launch();
@@ -1017,11 +1015,11 @@ static cudaError_t plane_lg_pair(int which, const cplx<T>* psi, int64_t ldpsi, c
   }
   const size_t sm = plane_lg_smem<T, N2, N3>(sp, plan);
   if (which == 0) {
-    if ((e = cudaFuncSetAttribute(k_plane_inv_lg<T, N2, N3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)))
+    if ((e = smem_limit(k_plane_inv_lg<T, N2, N3>, sm)))
       return e;
     k_plane_inv_lg<T, N2, N3><<<dim3(sp.nplane, nb), 256, sm, st>>>(psi, ldpsi, hb, hb_bs, sp, plan, tw); count_launch();
   } else {
-    if ((e = cudaFuncSetAttribute(k_plane_fwd_lg<T, N2, N3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)))
+    if ((e = smem_limit(k_plane_fwd_lg<T, N2, N3>, sm)))
       return e;
     k_plane_fwd_lg<T, N2, N3><<<dim3(sp.nplane, nb), 256, sm, st>>>(hb, hb_bs, sp, plan, tw, kin, psi, ldpsi, out,
                                                                     ldout); count_launch();
@@ -1607,7 +1605,7 @@ template <typename T, int N1, int TW>
 static cudaError_t launch_xline_tw(cplx<T>* hb, int64_t hb_bs, const T* vperm, const SphereDev& sp,
                                    const FftPlan& plan, int nb, cudaStream_t st) {
   const size_t sm = sizeof(cplx<T>) * (size_t)N1 * 32;
-  cudaError_t e = cudaFuncSetAttribute(k_xline_tw<T, N1, TW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  cudaError_t e = smem_limit(k_xline_tw<T, N1, TW>, sm);
   if (e) return e;
   if ((e = cudaFuncSetAttribute(k_xline_tw<T, N1, TW>, cudaFuncAttributePreferredSharedMemoryCarveout, 100))) return e;
   const int nyz = plan.n[1] * plan.n[2];
@@ -1624,7 +1622,7 @@ static cudaError_t launch_xline_twr(cplx<T>* hb, int64_t hb_bs, const T* vperm, 
   const int gx = (nyz + 31) / 32;
   cudaError_t e;
   if (staged && !multi) {
-    if ((e = cudaFuncSetAttribute(k_xline_tws<T, N1, TW, SW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)))
+    if ((e = smem_limit(k_xline_tws<T, N1, TW, SW>, sm)))
       return e;
     if ((e = cudaFuncSetAttribute(k_xline_tws<T, N1, TW, SW>, cudaFuncAttributePreferredSharedMemoryCarveout, 100)))
       return e;
@@ -1633,7 +1631,7 @@ static cudaError_t launch_xline_twr(cplx<T>* hb, int64_t hb_bs, const T* vperm, 
   }
   if (staged) {
     const size_t sm2 = 2 * sm;
-    if ((e = cudaFuncSetAttribute(k_xline_twd<T, N1, TW, SW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2)))
+    if ((e = smem_limit(k_xline_twd<T, N1, TW, SW>, sm2)))
       return e;
     if ((e = cudaFuncSetAttribute(k_xline_twd<T, N1, TW, SW>, cudaFuncAttributePreferredSharedMemoryCarveout, 100)))
       return e;
@@ -1645,14 +1643,14 @@ static cudaError_t launch_xline_twr(cplx<T>* hb, int64_t hb_bs, const T* vperm, 
     return cudaGetLastError();
   }
   if (!multi) {
-    if ((e = cudaFuncSetAttribute(k_xline_twr<T, N1, TW, SW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)))
+    if ((e = smem_limit(k_xline_twr<T, N1, TW, SW>, sm)))
       return e;
     if ((e = cudaFuncSetAttribute(k_xline_twr<T, N1, TW, SW>, cudaFuncAttributePreferredSharedMemoryCarveout, 100)))
       return e;
     k_xline_twr<T, N1, TW, SW><<<dim3(gx, nb), 32 * TW, sm, st>>>(hb, hb_bs, vperm, sp, plan, tw); count_launch();
     return cudaGetLastError();
   }
-  if ((e = cudaFuncSetAttribute(k_xline_twm<T, N1, TW, SW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)))
+  if ((e = smem_limit(k_xline_twm<T, N1, TW, SW>, sm)))
     return e;
   if ((e = cudaFuncSetAttribute(k_xline_twm<T, N1, TW, SW>, cudaFuncAttributePreferredSharedMemoryCarveout, 100)))
     return e;
@@ -2295,8 +2293,7 @@ static cudaError_t plane_wg_pair(int which, const cplx<T>* psi, int64_t ldpsi, c
         if constexpr (std::is_same<T, float>::value) {
           auto run = [&](auto rc) -> cudaError_t {  // 1 with P Z, 2 without
             constexpr int R = decltype(rc)::value;
-          if ((e = cudaFuncSetAttribute(k_plane_fwd_wgp<T, N2, N3, TW, R>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)))
+          if ((e = smem_limit(k_plane_fwd_wgp<T, N2, N3, TW, R>, sm)))
             return e;
           const int grid = grid_of((const void*)k_plane_fwd_wgp<T, N2, N3, TW, R>);
           k_plane_fwd_wgp<T, N2, N3, TW, R><<<grid, PW::THREADS, sm, st>>>(hb, hb_bs, sp, plan, tw, kin, psi,
@@ -2310,8 +2307,7 @@ static cudaError_t plane_wg_pair(int which, const cplx<T>* psi, int64_t ldpsi, c
           return cudaErrorNotSupported;
         }
       } else {
-        if ((e = cudaFuncSetAttribute(k_plane_fwd_wgp<T, N2, N3, TW, 0>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)))
+        if ((e = smem_limit(k_plane_fwd_wgp<T, N2, N3, TW, 0>, sm)))
           return e;
         const int grid = grid_of((const void*)k_plane_fwd_wgp<T, N2, N3, TW, false>);
         k_plane_fwd_wgp<T, N2, N3, TW, 0><<<grid, PW::THREADS, sm, st>>>(hb, hb_bs, sp, plan, tw, kin, psi,
@@ -2323,8 +2319,7 @@ static cudaError_t plane_wg_pair(int which, const cplx<T>* psi, int64_t ldpsi, c
     if (which == 0 && persist) {
       int nsm = 152, dev = 0, per = 1;
       if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-      if ((e = cudaFuncSetAttribute(k_plane_inv_wgp<T, N2, N3, TW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)sm)))
+      if ((e = smem_limit(k_plane_inv_wgp<T, N2, N3, TW>, sm)))
         return e;
       if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_plane_inv_wgp<T, N2, N3, TW>, PW::THREADS, sm) !=
               cudaSuccess || per < 1)
@@ -2335,8 +2330,7 @@ static cudaError_t plane_wg_pair(int which, const cplx<T>* psi, int64_t ldpsi, c
       return cudaGetLastError();
     }
     if (which == 0) {
-      if ((e = cudaFuncSetAttribute(k_plane_inv_wg<T, N2, N3, TW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)sm)))
+      if ((e = smem_limit(k_plane_inv_wg<T, N2, N3, TW>, sm)))
         return e;
       if ((e = cudaFuncSetAttribute(k_plane_inv_wg<T, N2, N3, TW>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                     100)))
@@ -2348,8 +2342,7 @@ static cudaError_t plane_wg_pair(int which, const cplx<T>* psi, int64_t ldpsi, c
         if constexpr (std::is_same<T, float>::value) {
           auto run = [&](auto rc) -> cudaError_t {  // 1 with P Z, 2 without
             constexpr int R = decltype(rc)::value;
-          if ((e = cudaFuncSetAttribute(k_plane_fwd_wg<T, N2, N3, TW, R>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)))
+          if ((e = smem_limit(k_plane_fwd_wg<T, N2, N3, TW, R>, sm)))
             return e;
           if ((e = cudaFuncSetAttribute(k_plane_fwd_wg<T, N2, N3, TW, R>,
                                         cudaFuncAttributePreferredSharedMemoryCarveout, 100)))
@@ -2364,8 +2357,7 @@ static cudaError_t plane_wg_pair(int which, const cplx<T>* psi, int64_t ldpsi, c
           return cudaErrorNotSupported;
         }
       } else {
-        if ((e = cudaFuncSetAttribute(k_plane_fwd_wg<T, N2, N3, TW, 0>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)))
+        if ((e = smem_limit(k_plane_fwd_wg<T, N2, N3, TW, 0>, sm)))
           return e;
         if ((e = cudaFuncSetAttribute(k_plane_fwd_wg<T, N2, N3, TW, 0>,
                                       cudaFuncAttributePreferredSharedMemoryCarveout, 100)))
@@ -2682,16 +2674,14 @@ static cudaError_t plane_rs_pair(int which, const cplx<T>* psi, int64_t ldpsi, c
     cudaError_t e;
     const dim3 grid(sp.nplane, nb);
     if (which == 0) {
-      if ((e = cudaFuncSetAttribute(k_plane_inv_rs<T, N2, N3, TW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)sm)))
+      if ((e = smem_limit(k_plane_inv_rs<T, N2, N3, TW>, sm)))
         return e;
       k_plane_inv_rs<T, N2, N3, TW><<<grid, PR::THREADS, sm, st>>>(psi, ldpsi, hb, hb_bs, sp, plan, tw); count_launch();
     } else if (rec) {
       if constexpr (kF32) {
           auto run = [&](auto rc) -> cudaError_t {  // 1 with P Z, 2 without
             constexpr int R = decltype(rc)::value;
-        if ((e = cudaFuncSetAttribute(k_plane_fwd_rs<T, N2, N3, TW, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)sm)))
+        if ((e = smem_limit(k_plane_fwd_rs<T, N2, N3, TW, R>, sm)))
           return e;
         k_plane_fwd_rs<T, N2, N3, TW, R><<<grid, PR::THREADS, sm, st>>>(hb, hb_bs, sp, plan, tw, kin, psi, ldpsi,
                                                                           out, ldout, *rec); count_launch();
@@ -2701,8 +2691,7 @@ static cudaError_t plane_rs_pair(int which, const cplx<T>* psi, int64_t ldpsi, c
           if (e) return e;
         }
     } else {
-      if ((e = cudaFuncSetAttribute(k_plane_fwd_rs<T, N2, N3, TW, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)sm)))
+      if ((e = smem_limit(k_plane_fwd_rs<T, N2, N3, TW, 0>, sm)))
         return e;
       k_plane_fwd_rs<T, N2, N3, TW, 0><<<grid, PR::THREADS, sm, st>>>(hb, hb_bs, sp, plan, tw, kin, psi, ldpsi,
                                                                          out, ldout, Pass3Rec{}); count_launch();
@@ -2738,7 +2727,7 @@ static cudaError_t launch_xline_tpl(cplx<T>* hb, int64_t hb_bs, const T* vperm, 
                                     const FftPlan& plan, int nb, cudaStream_t st) {
   const size_t sm = sizeof(cplx<T>) * (size_t)N1 * kTplX;
   if (sm > 227 * 1024) return cudaErrorNotSupported;
-  cudaError_t e = cudaFuncSetAttribute(k_xline_tpl<T, N1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  cudaError_t e = smem_limit(k_xline_tpl<T, N1>, sm);
   if (e) return e;
   if ((e = cudaFuncSetAttribute(k_xline_tpl<T, N1>, cudaFuncAttributePreferredSharedMemoryCarveout, 100))) return e;
   const int nyz = plan.n[1] * plan.n[2];
@@ -2777,13 +2766,13 @@ static cudaError_t plane_tpl_pair(int which, const cplx<T>* psi, int64_t ldpsi, 
     if (sm > 227 * 1024 || sp.max_rows > PT::THREADS * 4) return cudaErrorNotSupported;
     cudaError_t e;
     if (which == 0) {
-      if ((e = cudaFuncSetAttribute(k_plane_inv_tpl<T, N2, N3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)))
+      if ((e = smem_limit(k_plane_inv_tpl<T, N2, N3>, sm)))
         return e;
       if ((e = cudaFuncSetAttribute(k_plane_inv_tpl<T, N2, N3>, cudaFuncAttributePreferredSharedMemoryCarveout, 100)))
         return e;
       k_plane_inv_tpl<T, N2, N3><<<dim3(sp.nplane, nb), PT::THREADS, sm, st>>>(psi, ldpsi, hb, hb_bs, sp); count_launch();
     } else {
-      if ((e = cudaFuncSetAttribute(k_plane_fwd_tpl<T, N2, N3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)))
+      if ((e = smem_limit(k_plane_fwd_tpl<T, N2, N3>, sm)))
         return e;
       if ((e = cudaFuncSetAttribute(k_plane_fwd_tpl<T, N2, N3>, cudaFuncAttributePreferredSharedMemoryCarveout, 100)))
         return e;
@@ -2833,9 +2822,9 @@ cudaError_t launch_local_apply(const FftPlan& plan, const cplx<T>* tw, const Sph
   const size_t sm1 = plane_smem<T>(plan, sp, cz);
   const size_t sm2 = sizeof(cplx<T>) * (size_t)plan.n[0] * lyz;
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(k_plane_inv<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1))) return e;
-  if ((e = cudaFuncSetAttribute(k_plane_fwd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1))) return e;
-  if ((e = cudaFuncSetAttribute(k_xline<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2))) return e;
+  if ((e = smem_limit(k_plane_inv<T>, sm1))) return e;
+  if ((e = smem_limit(k_plane_fwd<T>, sm1))) return e;
+  if ((e = smem_limit(k_xline<T>, sm2))) return e;
   const int64_t hb_bs = (int64_t)sp.nplane * plan.n[1] * plan.n[2];
   const int nyz = plan.n[1] * plan.n[2];
   // one-thread-per-line kernels: complex64 only (a complex128 line per thread needs twice
@@ -3025,7 +3014,7 @@ cudaError_t launch_local_apply_rec(const FftPlan& plan, const float2* tw, const 
     }
     if (e == cudaErrorNotSupported) {
       (void)cudaGetLastError();
-      if ((e = cudaFuncSetAttribute(k_xline<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2))) return e;
+      if ((e = smem_limit(k_xline<T>, sm2))) return e;
       k_xline<T><<<dim3((nyz + lyz - 1) / lyz, nb), kThreads, sm2, st>>>(hb, hb_bs, vperm, sp, plan, tw, lyz); count_launch();
       e = cudaGetLastError();
     }
@@ -3147,7 +3136,7 @@ static cudaError_t launch_xdens_wg(const cplx<T>* hba, const cplx<T>* hbb, int64
                                    cudaStream_t st) {
   constexpr int TW = 4;
   const size_t sm = sizeof(cplx<T>) * (size_t)N1 * 32 * (hbb ? 2 : 1);
-  cudaError_t e = cudaFuncSetAttribute(k_xdens_wg<T, N1, TW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  cudaError_t e = smem_limit(k_xdens_wg<T, N1, TW>, sm);
   if (e) return e;
   if ((e = cudaFuncSetAttribute(k_xdens_wg<T, N1, TW>, cudaFuncAttributePreferredSharedMemoryCarveout, 100))) return e;
   const int nyz = plan.n[1] * plan.n[2];
@@ -3192,8 +3181,8 @@ cudaError_t launch_density(const FftPlan& plan, const cplx<T>* tw, const SphereD
   const size_t sm1 = plane_smem<T>(plan, sp, cz);
   const size_t sm2 = sizeof(cplx<T>) * (size_t)plan.n[0] * lyz * 2;
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(k_plane_inv<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1))) return e;
-  if ((e = cudaFuncSetAttribute(k_xline_density<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2))) return e;
+  if ((e = smem_limit(k_plane_inv<T>, sm1))) return e;
+  if ((e = smem_limit(k_xline_density<T>, sm2))) return e;
   const int64_t hb_bs = (int64_t)sp.nplane * plan.n[1] * plan.n[2];
   const int nyz = plan.n[1] * plan.n[2];
   cplx<T>* hbb = b ? hb + hb_bs * band_batch : nullptr;

@@ -164,7 +164,7 @@ cudaError_t la_trinv_lower_keep(const double2* L, int64_t lda, int n, double2* X
   k_keep_transpose<<<g, b, 0, st>>>(L, lda, n, tmp); count_launch();
   const int wpb = 4;
   const size_t sm = sizeof(double2) * (size_t)n * wpb;
-  cudaError_t e = cudaFuncSetAttribute(k_keep_trinv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  cudaError_t e = smem_limit(k_keep_trinv, sm);
   if (e) return e;
   k_keep_trinv<<<(n + wpb - 1) / wpb, 32 * wpb, sm, st>>>(tmp, n, X, ldx); count_launch();
   return cudaGetLastError();

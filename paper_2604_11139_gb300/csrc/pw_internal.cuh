@@ -361,4 +361,15 @@ void prof_begin(pw_ctx* c, int cls);
 void prof_end(pw_ctx* c, int cls);
 int set_error(int status, const char* fmt, ...);
 int cuda_status(cudaError_t e, const char* where);
+
+// Before a launch with `bytes` of dynamic shared memory.  A kernel's limit is one value for the whole
+// process: set to each launch's own size, it would be lowered by another thread's smaller call between
+// this one and the launch, which then fails.  So every call sets the same limit, the most a kernel can
+// have beside its static shared memory (227 KB without any).  Up to 48 KB in all (at most 3 KB are
+// static) need none.
+template <typename F> cudaError_t smem_limit(F* f, size_t bytes, size_t limit = 227 * 1024) {
+  if (bytes > limit) return cudaErrorInvalidValue;
+  if (bytes <= 45 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute((const void*)f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit);
+}
 }  // namespace pw
