@@ -2881,9 +2881,9 @@ cudaError_t launch_local_apply(const FftPlan& plan, const cplx<T>* tw, const Sph
     if (e == cudaErrorNotSupported) {
       (void)cudaGetLastError();
       k_plane_inv<T><<<dim3(sp.nplane, nb), kThreads, sm1, st>>>(psi + b0 * ldpsi, ldpsi, hb, hb_bs, sp, plan, tw, cz); count_launch();
-    } else if (e != cudaSuccess) {
-      return e;
+      e = cudaGetLastError();
     }
+    if (e != cudaSuccess) return e;
     prof_end(prof, PW_PROF_PLANE_INV);
     prof_begin(prof, PW_PROF_XLINE);
     e = cudaErrorNotSupported;
@@ -2910,9 +2910,9 @@ cudaError_t launch_local_apply(const FftPlan& plan, const cplx<T>* tw, const Sph
     if (e == cudaErrorNotSupported) {
       (void)cudaGetLastError();
       k_xline<T><<<dim3((nyz + lyz - 1) / lyz, nb), kThreads, sm2, st>>>(hb, hb_bs, vperm, sp, plan, tw, lyz); count_launch();
-    } else if (e != cudaSuccess) {
-      return e;
+      e = cudaGetLastError();
     }
+    if (e != cudaSuccess) return e;
     prof_end(prof, PW_PROF_XLINE);
     prof_begin(prof, PW_PROF_PLANE_FWD);
     e = cudaErrorNotSupported;
@@ -2939,9 +2939,9 @@ cudaError_t launch_local_apply(const FftPlan& plan, const cplx<T>* tw, const Sph
       (void)cudaGetLastError();
       k_plane_fwd<T><<<dim3(sp.nplane, nb), kThreads, sm1, st>>>(hb, hb_bs, sp, plan, tw, cz, kin,
                                                                   psi + b0 * ldpsi, ldpsi, out + b0 * ldout, ldout); count_launch();
-    } else if (e != cudaSuccess) {
-      return e;
+      e = cudaGetLastError();
     }
+    if (e != cudaSuccess) return e;
     prof_end(prof, PW_PROF_PLANE_FWD);
   }
   return cudaGetLastError();

@@ -250,13 +250,17 @@ Epi<T> epi(int mode, cplx<T>* out, int64_t ldo, T alpha = 1) {
   return e;
 }
 
-// Bands per FFT batch: half-box planes near fft_batch_bytes (complex64 384 MB, complex128 512 MB
-// unless tuned), a few large launches.
-int band_batch(const pw_ctx* ctx, int nband, size_t elem = 16) {
+// Bands per FFT batch: half-box planes near `target` bytes, a few large launches; a launch has a
+// band per blockIdx.y, of which there are 65535.
+constexpr size_t kMaxBandBatch = 65535;
+int bands_within(const pw_ctx* ctx, int nband, size_t elem, size_t target) {
   const size_t per = (size_t)ctx->sp.nplane * ctx->n[1] * ctx->n[2] * elem;
-  const size_t target = ctx->fft_batch_bytes[elem == 8 ? 0 : 1];
-  int bb = (int)std::max<size_t>(1, target / std::max<size_t>(per, 1));
-  return std::max(1, std::min(bb, nband));
+  const size_t most = std::min<size_t>(kMaxBandBatch, std::max(nband, 1));
+  return (int)std::min(most, std::max<size_t>(1, target / std::max<size_t>(per, 1)));
+}
+// the batch of the context's configuration (complex64 384 MB, complex128 512 MB unless tuned)
+int band_batch(const pw_ctx* ctx, int nband, size_t elem = 16) {
+  return bands_within(ctx, nband, elem, ctx->fft_batch_bytes[elem == 8 ? 0 : 1]);
 }
 
 // ---------------------------------------------------------------------------
@@ -2054,7 +2058,7 @@ PW_API int pw_autotune(pw_ctx* ctx, int nband, int precision, double* best_ms) {
   WS(xout, unsigned char, WS_Y2, elem * (size_t)ctx->npw * nband);
   CU_TRY(cudaMemsetAsync(xin, 0, elem * (size_t)ctx->npw * nband, st), "autotune input");
   size_t max_hb = 0;
-  for (size_t c : cand) max_hb = std::max(max_hb, std::min<size_t>(std::max<size_t>(c / std::max<size_t>(per, 1), 1), nband) * per);
+  for (size_t c : cand) max_hb = std::max(max_hb, bands_within(ctx, nband, elem, c) * per);
   WS(hb, unsigned char, WS_HB, max_hb);
   // events and the profiling switch are restored on every exit path
   struct Guard {
@@ -2075,7 +2079,7 @@ PW_API int pw_autotune(pw_ctx* ctx, int nband, int precision, double* best_ms) {
   int best_v = ctx->fft_variant[slot];
   std::vector<std::pair<float, int>> form_times;  // (time, variant) of the form sweep
   auto consider = [&](size_t c, int v, int reps = 5) -> int {
-    const int bb = (int)std::max<size_t>(1, std::min<size_t>(c / std::max<size_t>(per, 1), nband));
+    const int bb = bands_within(ctx, nband, elem, c);
     if (c != cand[0] && bb * per > c && bb == 1) return PW_OK;
     ctx->fft_variant[slot] = v;
     float tot = 1e30f;  // the fastest of the timed runs (after a warm-up) resists noise best
