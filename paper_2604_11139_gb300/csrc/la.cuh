@@ -36,6 +36,8 @@ constexpr int la_lz_blocks = 152;
 cudaError_t la_lanczos(const double2* v0, int n, int steps, double2* v, double2* vprev, double2* w, double* ab,
                        double* bound, double* part, ApplyFn apply, void* ctx, cudaStream_t st);
 cudaError_t la_to_c64(const double2* a, int64_t lda, float2* b, int64_t ldb, int n, int m, cudaStream_t st);
+// b (n x n) <- a times the power of two that brings its largest component into [1, 2); top: one word
+cudaError_t la_to_c64_scaled(const double2* a, float2* b, int n, unsigned* top, cudaStream_t st);
 cudaError_t la_to_c128(const float2* a, int64_t lda, double2* b, int64_t ldb, int n, int m, cudaStream_t st);
 // LOBPCG: W = K (HX - lam SX) with the Teter-Payne-Allan preconditioner, rn = residual norms
 cudaError_t la_lob_resid(const double2* HX, const double2* SX, const double2* X, int64_t ld, int npw, int m,

@@ -829,6 +829,30 @@ cudaError_t la_to_c64(const double2* a, int64_t lda, float2* b, int64_t ldb, int
   k_c128_to_c64<<<(unsigned)((t + 255) / 256), 256, 0, st>>>(a, lda, b, ldb, n, m); count_launch();
   return cudaGetLastError();
 }
+// exponent field of the largest component of a (n entries)
+__global__ void __launch_bounds__(256) k_top_exp(const double2* a, int64_t n, unsigned* top) {
+  unsigned m = 0;
+  for (int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
+    const double2 v = a[i];
+    m = max(m, max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu));
+  }
+  m = __reduce_max_sync(0xffffffffu, m >> 20);
+  if ((threadIdx.x & 31) == 0) atomicMax(top, m);
+}
+__global__ void __launch_bounds__(256) k_to_c64_scaled(const double2* a, float2* b, int64_t n, const unsigned* top) {
+  const int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x;
+  if (i >= n) return;
+  const int s = 1023 - (int)*top;
+  b[i] = make_float2((float)scalbn(a[i].x, s), (float)scalbn(a[i].y, s));
+}
+cudaError_t la_to_c64_scaled(const double2* a, float2* b, int n, unsigned* top, cudaStream_t st) {
+  const int64_t t = (int64_t)n * n;
+  const cudaError_t e = cudaMemsetAsync(top, 0, sizeof(unsigned), st);
+  if (e) return e;
+  k_top_exp<<<(unsigned)std::min<int64_t>(64, (t + 255) / 256), 256, 0, st>>>(a, t, top); count_launch();
+  k_to_c64_scaled<<<(unsigned)((t + 255) / 256), 256, 0, st>>>(a, b, t, top); count_launch();
+  return cudaGetLastError();
+}
 cudaError_t la_to_c128(const float2* a, int64_t lda, double2* b, int64_t ldb, int n, int m, cudaStream_t st) {
   const int64_t t = (int64_t)n * m;
   if (t <= 0) return cudaSuccess;

@@ -982,7 +982,9 @@ int eigh_impl(pw_ctx* ctx, double2* A, int n, double2* U, double* eig, double2* 
     return PW_OK;
   };
   CU_TRY(cudaMemsetAsync(flag, 0, sizeof(int), st), "flag reset");
-  CU_TRY(la_to_c64(A, n, A32, n, n, n, st), "eig: to c64");
+  // the rotations do not depend on the scale of A, which may lie beyond FP32's range
+  if (keep) CU_TRY(la_to_c64(A, n, A32, n, n, n, st), "eig: to c64");
+  else CU_TRY(la_to_c64_scaled(A, A32, n, (unsigned*)flag + 1, st), "eig: to c64");
   int sw32 = 0, sw64 = 0;
   PW_TRY(la_jacobi_rotate32(A32, n, V32, w32, norms, st, 30, 1e-6, &sw32));
   CU_TRY(la_to_c128(V32, n, V, n, n, n, st), "eig: to c128");
