@@ -1,10 +1,12 @@
-// Factorisations and Lanczos steps of the FP64 pw_chebfi_solve, in one fixed order of operations.
+// Factorisations and Lanczos steps of the FP64 solves (pw_chebfi_solve, pw_batch_chebfi_solve), in one
+// fixed order of operations.
 //
 // The phase of a Ritz vector is a product of the phases of all the elements that the Jacobi rounds
 // met, the last of them at rounding level: another order of sums anywhere before it, however exact,
 // turns the vectors by phases of order one.  A program that keeps vectors of FP64 solves (or compares
-// them) sees the same ones only with the same operations, so this call runs the FP64 transforms, these
-// kernels and the plain Jacobi (pw_ctx::keep64).  Every other call returns the faster kernels' results:
+// them) sees the same ones only with the same operations, so these calls run the FP64 transforms, these
+// kernels and the plain Jacobi (pw_ctx::keep64), and a k-point has the same vectors alone and in a
+// batch.  Every other call returns the faster kernels' results:
 // the densities, energies, residuals and gradients that are made from Ritz vectors do not depend on
 // the phases.
 #include <math.h>

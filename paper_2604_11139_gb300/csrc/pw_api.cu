@@ -1684,6 +1684,21 @@ int gemm_nsplit(int m, int n, int k) { return nsplit_for(m, n, k); }
 }  // namespace api
 }  // namespace pw
 
+// FP64 solves, of one k-point and of a batch, keep one order of operations and with it the phases of
+// their vectors (la_keep.cu)
+namespace {
+struct Keep64 {
+  pw_ctx* const* c;
+  int n;
+  Keep64(pw_ctx* const* ctxs, int count, int precision) : c(ctxs), n(count) {
+    for (int i = 0; i < n; ++i) c[i]->keep64 = precision == PW_FP64;
+  }
+  ~Keep64() {
+    for (int i = 0; i < n; ++i) c[i]->keep64 = false;
+  }
+};
+}  // namespace
+
 // ---------------------------------------------------------------------------
 // k-point batches: every k-point's filter captured into one CUDA graph
 // ---------------------------------------------------------------------------
@@ -1696,12 +1711,14 @@ struct pw_batch {
   std::vector<cudaEvent_t> ev;
   double* dev_ce = nullptr;  // {c, e} per k-point
   std::vector<double> host_ce;
-  cudaGraph_t graph = nullptr;
-  cudaGraphExec_t exec = nullptr;
-  std::vector<void*> key_psi;
-  std::vector<int64_t> key_ld;
-  std::vector<uint64_t> key_gen;
-  int key_nband = -1, key_degree = -1, key_prec = -1;
+  struct Graph {
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    std::vector<void*> key_psi;
+    std::vector<int64_t> key_ld;
+    std::vector<uint64_t> key_gen;
+    int key_nband = -1, key_degree = -1, key_prec = -1;
+  } graphs[2];  // of the filters, and of those inside FP64 solves (pw_ctx::keep64)
   std::vector<void*> y32;  // complex64 copies for the mixed solve
   std::vector<size_t> y32_bytes;
   bool poisoned = false;
@@ -1711,11 +1728,11 @@ namespace {
 
 constexpr int kBatchStreams = 4;
 
-void batch_free_graph(pw_batch* bt) {
-  if (bt->exec) cudaGraphExecDestroy(bt->exec);
-  if (bt->graph) cudaGraphDestroy(bt->graph);
-  bt->exec = nullptr;
-  bt->graph = nullptr;
+void batch_free_graph(pw_batch::Graph& gr) {
+  if (gr.exec) cudaGraphExecDestroy(gr.exec);
+  if (gr.graph) cudaGraphDestroy(gr.graph);
+  gr.exec = nullptr;
+  gr.graph = nullptr;
 }
 
 int batch_run_one(pw_batch* bt, int k, void* psi, int64_t ld, int nband, int degree, int precision) {
@@ -1728,17 +1745,18 @@ int batch_run_one(pw_batch* bt, int k, void* psi, int64_t ld, int nband, int deg
 int batch_filter_body(pw_batch* bt, void* const* psi, const int64_t* ld, int nband, int degree, int precision) {
   const int nk = (int)bt->ctx.size();
   cudaError_t e;
-  bool same = bt->exec && bt->key_nband == nband && bt->key_degree == degree && bt->key_prec == precision;
+  pw_batch::Graph& gr = bt->graphs[bt->ctx[0]->keep64];
+  bool same = gr.exec && gr.key_nband == nband && gr.key_degree == degree && gr.key_prec == precision;
   for (int k = 0; same && k < nk; ++k)
-    same = bt->key_psi[k] == psi[k] && bt->key_ld[k] == ld[k] && bt->key_gen[k] == bt->ctx[k]->ws_gen;
+    same = gr.key_psi[k] == psi[k] && gr.key_ld[k] == ld[k] && gr.key_gen[k] == bt->ctx[k]->ws_gen;
   if (same) {
-    e = cudaGraphLaunch(bt->exec, bt->cap);
+    e = cudaGraphLaunch(gr.exec, bt->cap);
     if (e != cudaSuccess) { bt->poisoned = true; return cuda_status(e, "batch graph launch"); }
     return PW_OK;
   }
   // first call for this shape: run eagerly (allocates every workspace), then capture the
   // same launches, fanned out over kBatchStreams streams, for the following calls
-  batch_free_graph(bt);
+  batch_free_graph(gr);
   std::vector<cudaStream_t> saved(nk);
   for (int k = 0; k < nk; ++k) {
     if (bt->ctx[k]->prof_on) return set_error(PW_EINVAL, "disable profiling on batched contexts");
@@ -1767,9 +1785,9 @@ int batch_filter_body(pw_batch* bt, void* const* psi, const int64_t* ld, int nba
     cudaGraph_t g = nullptr;
     const cudaError_t e2 = cudaStreamEndCapture(bt->cap, &g);
     if (st == PW_OK && e2 == cudaSuccess && g) {
-      bt->graph = g;
-      e = cudaGraphInstantiate(&bt->exec, g, 0);
-      if (e != cudaSuccess) { batch_free_graph(bt); st = cuda_status(e, "batch graph instantiate"); }
+      gr.graph = g;
+      e = cudaGraphInstantiate(&gr.exec, g, 0);
+      if (e != cudaSuccess) { batch_free_graph(gr); st = cuda_status(e, "batch graph instantiate"); }
     } else {
       if (g) cudaGraphDestroy(g);
       if (st == PW_OK) st = cuda_status(e2 == cudaSuccess ? cudaErrorStreamCaptureInvalidated : e2, "batch capture");
@@ -1779,13 +1797,13 @@ int batch_filter_body(pw_batch* bt, void* const* psi, const int64_t* ld, int nba
   }
   for (int k = 0; k < nk; ++k) bt->ctx[k]->stream = saved[k];
   if (st != PW_OK) return st;
-  bt->key_psi.assign(psi, psi + nk);
-  bt->key_ld.assign(ld, ld + nk);
-  bt->key_gen.resize(nk);
-  for (int k = 0; k < nk; ++k) bt->key_gen[k] = bt->ctx[k]->ws_gen;
-  bt->key_nband = nband;
-  bt->key_degree = degree;
-  bt->key_prec = precision;
+  gr.key_psi.assign(psi, psi + nk);
+  gr.key_ld.assign(ld, ld + nk);
+  gr.key_gen.resize(nk);
+  for (int k = 0; k < nk; ++k) gr.key_gen[k] = bt->ctx[k]->ws_gen;
+  gr.key_nband = nband;
+  gr.key_degree = degree;
+  gr.key_prec = precision;
   return PW_OK;
 }
 
@@ -1961,12 +1979,7 @@ PW_API int pw_chebfi_solve(pw_ctx* ctx, void* psi_v, int64_t ldpsi, int nband, i
   if (nband == 0) return PW_OK;
   if (!eig) return set_error(PW_EINVAL, "eig is NULL");
   if (precision != PW_FP64 && precision != PW_MIXED) return set_error(PW_EINVAL, "unknown precision");
-  // the FP64 form keeps its order of operations, and with it the phases of its vectors (la_keep.cu)
-  struct Keep {
-    pw_ctx* c;
-    ~Keep() { c->keep64 = false; }
-  } keep{ctx};
-  ctx->keep64 = precision == PW_FP64;
+  const Keep64 keep(&ctx, 1, precision);
   double2* psi = (double2*)psi_v;
   double rqmin = 0, a = 0, upper = 0;
   if (precision == PW_MIXED) {
@@ -2328,7 +2341,7 @@ PW_API int pw_batch_create(pw_ctx* const* ctxs, int nk, void* stream, pw_batch**
 PW_API int pw_batch_destroy(pw_batch* bt) {
   if (!bt) return PW_OK;
   if (bt->cap) cudaStreamSynchronize(bt->cap);
-  batch_free_graph(bt);
+  for (auto& gr : bt->graphs) batch_free_graph(gr);
   if (bt->cap) cudaStreamDestroy(bt->cap);
   if (bt->ev_in) cudaEventDestroy(bt->ev_in);
   if (bt->ev_out) cudaEventDestroy(bt->ev_out);
@@ -2364,6 +2377,7 @@ PW_API int pw_batch_chebfi_solve(pw_batch* bt, void* const* psi, const int64_t* 
     PW_TRY(check_block(bt->ctx[k], psi[k], ld[k], nband));
   }
   if (nband == 0) return PW_OK;
+  const Keep64 keep(bt->ctx.data(), nk, precision);
   std::vector<double> a(nk), b(nk);
   for (int k = 0; k < nk; ++k) {
     pw_ctx* ctx = bt->ctx[k];

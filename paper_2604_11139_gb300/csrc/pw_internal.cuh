@@ -333,7 +333,7 @@ struct pw_ctx {
   // column-slice plane kernels (plane form 3), which fall back to line groups where they do
   // not apply (1.2x the line-group form on the 120^3 box)
   int fft_variant[2] = {8 + 3 * pw::kFormStride, 3 * pw::kFormStride};
-  bool keep64 = false;  // inside an FP64 pw_chebfi_solve: fixed order of operations (la_keep.cu)
+  bool keep64 = false;  // inside an FP64 solve: fixed order of operations (la_keep.cu)
   int last_sweeps = 0;  // Jacobi sweeps of the last Rayleigh-Ritz step
   // K splits of the mixed projection GEMM per column count, chosen by pw_autotune (columns ->
   // splits); other column counts use the whole-waves rule
