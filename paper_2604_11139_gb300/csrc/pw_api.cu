@@ -2172,8 +2172,10 @@ PW_API int pw_autotune(pw_ctx* ctx, int nband, int precision, double* best_ms) {
     best_v = fv;
     best_c = c2;
     ctx->fft_variant[slot] = fv;
-  } else {
-    // complex128: line-group planes or sphere rows + column slices (x-line form fixed)
+  } else if (!fx::covers(ctx->plan)) {
+    // complex128: line-group planes or sphere rows + column slices (x-line form fixed).  Boxes of the
+    // fixed-point passes keep their form: the applies timed here do not use it, and an FP64 solve,
+    // which does, keeps its order of operations.
     PW_TRY(consider(c1, 0));
     PW_TRY(consider(c1, 3 * kFormStride));
   }
