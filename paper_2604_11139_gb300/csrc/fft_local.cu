@@ -2807,6 +2807,25 @@ static size_t plane_smem(const FftPlan& plan, const SphereDev& sp, int cz) {
   return sizeof(cplx<T>) * ((size_t)sp.max_rows * plan.n[2] + (size_t)cz * (plan.n[1] + 1));
 }
 
+// boxes with line-group plane kernels: faster there than the kernels for any two-stage plan
+static bool plane_lg_covers(const FftPlan& plan) {
+  return plane_wg_covers(plan);  // the same boxes
+}
+
+// complex64 planes of boxes without kernels of their own: whether nb bands take the block-wide passes
+// (one launch, a CTA per plane and band) instead of those for any two-stage plan (z- and y-lines in two
+// launches, about 21 us a pass however few the lines).  While every plane has a place on the chip at
+// once, two per SM or four small ones, a block-wide pass takes 10 us (18^2 points), 13 (32^2), 18 (54 x
+// 60), 23 (72 x 75); the next plane on an SM costs 30 to 50% more.  The recurrence in pass 3 (`rec`) is
+// worth about 9 us a step, so a filter changes over earlier.  us for a 6-step filter with the block-wide
+// planes and without: 25 x 27 x 30, 8 bands 442 and 502, 32 bands (352 planes) 570 and 519; 54 x 54 x 60,
+// 1 band 559 and 577.
+static bool planes_block_wide(const FftPlan& plan, const SphereDev& sp, int nb, bool rec) {
+  if (plane_lg_covers(plan)) return false;
+  const int64_t planes = (int64_t)sp.nplane * nb, points = (int64_t)plan.n[1] * plan.n[2];
+  return planes <= (points <= 900 ? 4 : 2) * 152 && points <= (rec ? 3300 : 5400);
+}
+
 template <typename T>
 cudaError_t launch_local_apply(const FftPlan& plan, const cplx<T>* tw, const SphereDev& sp,
                                const T* vperm, const T* kin, const cplx<T>* psi, int64_t ldpsi,
@@ -2860,6 +2879,7 @@ cudaError_t launch_local_apply(const FftPlan& plan, const cplx<T>* tw, const Sph
   const bool lines = fl::covers(plan);
   for (int b0 = 0; b0 < nband; b0 += band_batch) {
     const int nb = min(band_batch, nband - b0);
+    const bool plane_lines = lines && !planes_block_wide(plan, sp, nb, false);
     prof_begin(prof, PW_PROF_PLANE_INV);
     e = cudaErrorNotSupported;
     if constexpr (std::is_same<T, float>::value) {
@@ -2873,7 +2893,7 @@ cudaError_t launch_local_apply(const FftPlan& plan, const cplx<T>* tw, const Sph
       e = plane_lg<T>(0, psi + b0 * ldpsi, ldpsi, hb, hb_bs, sp, plan, tw, kin, nullptr, 0, nb, st);
     }
     if constexpr (std::is_same<T, float>::value) {
-      if (e == cudaErrorNotSupported && lines) {
+      if (e == cudaErrorNotSupported && plane_lines) {
         (void)cudaGetLastError();
         e = fl::inverse_planes(plan, tw, sp, psi + b0 * ldpsi, ldpsi, hb, hb_bs, nb, st);
       }
@@ -2929,7 +2949,7 @@ cudaError_t launch_local_apply(const FftPlan& plan, const cplx<T>* tw, const Sph
       e = plane_lg<T>(1, psi + b0 * ldpsi, ldpsi, hb, hb_bs, sp, plan, tw, kin, out + b0 * ldout, ldout, nb, st);
     }
     if constexpr (std::is_same<T, float>::value) {
-      if (e == cudaErrorNotSupported && lines) {
+      if (e == cudaErrorNotSupported && plane_lines) {
         (void)cudaGetLastError();
         e = fl::forward_planes(plan, tw, sp, kin, hb, hb_bs, psi + b0 * ldpsi, ldpsi, out + b0 * ldout, ldout, nb, st,
                                nullptr);
@@ -2952,16 +2972,11 @@ static bool plane_rs_covers(const FftPlan& plan) {
   return (n2 == 64 && n3 == 64) || (n2 == 72 && n3 == 90) || (n2 == 96 && n3 == 96) || (n2 == 120 && n3 == 120);
 }
 
-// boxes with line-group plane kernels: faster there than the kernels for any two-stage plan
-static bool plane_lg_covers(const FftPlan& plan) {
-  return plane_wg_covers(plan);  // the same boxes
-}
-
-bool local_apply_rec_supported(const FftPlan& plan, const ::pw_ctx* prof) {
+bool local_apply_rec_supported(const FftPlan& plan, const SphereDev& sp, int nband, const ::pw_ctx* prof) {
   if (!prof) return false;
   const int pf = prof->fft_variant[0] / kFormStride;
   return ((pf == 2 || pf == 6) && plane_wg_covers(plan)) || (pf == 3 && plane_rs_covers(plan)) ||
-         ((pf == 4 || pf == 5) && plane_wg_covers(plan) && plane_rs_covers(plan)) || (pf >= 2 && fl::covers(plan) && !plane_lg_covers(plan));
+         ((pf == 4 || pf == 5) && plane_wg_covers(plan) && plane_rs_covers(plan)) || (pf >= 2 && fl::covers(plan) && !plane_lg_covers(plan) && !planes_block_wide(plan, sp, nband, true));
 }
 
 cudaError_t launch_local_apply_rec(const FftPlan& plan, const float2* tw, const SphereDev& sp, const float* vperm,
@@ -2969,7 +2984,7 @@ cudaError_t launch_local_apply_rec(const FftPlan& plan, const float2* tw, const 
                                    int64_t ldout, float2* hb, int band_batch, cudaStream_t st, ::pw_ctx* prof,
                                    const Pass3Rec& rec) {
   using T = float;
-  if (!local_apply_rec_supported(plan, prof)) return cudaErrorNotSupported;
+  if (!local_apply_rec_supported(plan, sp, nband, prof)) return cudaErrorNotSupported;
   if (nband <= 0) return cudaSuccess;
   int xf = prof->fft_variant[0] % kFormStride;
   const float* vperm_x = vperm;

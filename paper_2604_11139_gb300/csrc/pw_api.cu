@@ -661,7 +661,7 @@ int filter_impl(pw_ctx* ctx, cplx<T>* psi, int64_t ldpsi, int nband, int degree,
   // the bf16 split of Y_{k+1} fused into pass 3 (fewer block reads than the recurrence in
   // the back-projection epilogue)
   if constexpr (kMixed) {
-    if (np > 0 && !ctx->has_q && local_apply_rec_supported(ctx->plan, ctx)) {
+    if (np > 0 && !ctx->has_q && local_apply_rec_supported(ctx->plan, ctx->sp, nband, ctx)) {
       WS(PZ, C, WS_PZ, (size_t)npw * nband);
       for (int k = 0; k < degree; ++k) {
         C* cur = buf[k % 3];
@@ -722,7 +722,7 @@ int filter_impl(pw_ctx* ctx, cplx<T>* psi, int64_t ldpsi, int nband, int degree,
     // projection takes (512 bands on 120^3, 12 steps: the pass over W took 4.6 ms, pass 3 2.2 ms longer)
     bool pieces_done = false;
     if constexpr (kMixed) {
-      if (shadow && local_apply_rec_supported(ctx->plan, ctx)) {
+      if (shadow && local_apply_rec_supported(ctx->plan, ctx->sp, nband, ctx)) {
         Pass3Rec rec{};
         rec.alpha = 1.f;
         rec.split = ys;

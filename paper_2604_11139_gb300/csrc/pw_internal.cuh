@@ -207,7 +207,7 @@ cudaError_t launch_local_apply_rec(const FftPlan& plan, const float2* tw, const 
                                    const float* kin, const float2* psi, int64_t ldpsi, int nband, float2* out,
                                    int64_t ldout, float2* hb, int band_batch, cudaStream_t st, ::pw_ctx* prof,
                                    const Pass3Rec& rec);
-bool local_apply_rec_supported(const FftPlan& plan, const ::pw_ctx* prof);
+bool local_apply_rec_supported(const FftPlan& plan, const SphereDev& sp, int nband, const ::pw_ctx* prof);
 
 template <typename T>
 cudaError_t launch_density(const FftPlan& plan, const cplx<T>* tw, const SphereDev& sp,
