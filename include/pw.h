@@ -400,8 +400,12 @@ enum pw_prof_class {
  * For PW_MIXED the bare-apply ranking is then checked inside two steps of the filter itself:
  * every plane form with the best x-line form, and the runner-up x-line form with the best
  * plane form; the fastest there is kept.
- * PW_FP64 tunes the plane form only (0 or 3, variant 0 or 48; its x-line form is fixed).
- * Forms other than 0 cover box lengths with two-stage radix plans.  Keeps the fastest for
+ * PW_FP64: where every box length has a two-stage radix plan up to 256 the complex128 passes
+ * run in 64-bit block fixed point and only the batch size is tuned; the plane form, which
+ * FP64 solves use there, is left alone (another one turns their vectors by phases).
+ * Elsewhere the plane form (0 or 3, variant 0 or 48; the x-line form is fixed) is tuned too.
+ * Complex64 forms other than 0 cover box lengths with two-stage radix plans; on boxes without
+ * kernels of their own all plane forms from 2 on run the same kernels.  Keeps the fastest for
  * `precision` in the context.  Synchronises the stream; *best_ms (may be NULL) receives
  * the best time of one apply. */
 PW_API int pw_autotune(pw_ctx* ctx, int nband, int precision, double* best_ms);
@@ -410,9 +414,13 @@ PW_API int pw_autotune(pw_ctx* ctx, int nband, int precision, double* best_ms);
  * other column counts use the rule. */
 /* Reads (*batch_bytes, *variant; either pointer may be NULL) and then, for arguments
  * >= 0, sets the FFT configuration of `precision`: bytes of half-box planes per band
- * batch (>= 1 band is always used) and the pass-kernel forms (as for
- * pw_autotune; non-zero forms apply to PW_MIXED only and fall back to 0 for box
- * lengths they do not cover).  Pass -1 to leave a field unchanged. */
+ * batch (1 to 65535 bands are used) and the pass-kernel forms (as for pw_autotune; forms fall
+ * back for box lengths they do not cover; for PW_FP64 variants 0 and 48, which concern FP64
+ * solves and boxes without two-stage plans).  Pass -1 to leave a field unchanged.
+ * Defaults: PW_MIXED 384 MB and variant 56, PW_FP64 512 MB and variant 48.  A context keeps the
+ * larger of the buffers it has used, at most the batch size or the planes of its largest block
+ * (every context of a batch its own); a smaller batch size set before the first call costs some
+ * speed and holds less. */
 PW_API int pw_fft_config(pw_ctx* ctx, int precision, int64_t set_batch_bytes, int set_variant,
                          int64_t* batch_bytes, int* variant);
 
@@ -429,8 +437,10 @@ PW_API int pw_tc_config(pw_ctx* ctx, int set_pieces, int* pieces);
  * power of two and cut into seven 7-bit integer digits; the 28 digit products with the seven
  * leading weights summed exactly in FP32 per 256-wide K chunk, combined in 64-bit integers and
  * accumulated in FP64; error per product below 2^-44 of the row and column maxima), 0 as DFMA
- * GEMMs.  Products with at most 4 columns (matrix-vector forms) and the M x M x M products of
- * the subspace step always use DFMA. */
+ * GEMMs.  The products of the differentiation form from 2^25 complex products on and those of the
+ * eigensolver's rotations above 160 columns take eight digits (below 2^-51).  Products below 2^22
+ * complex products or with at most 4 columns (matrix-vector forms) and the other M x M x M
+ * products of the subspace step always use DFMA. */
 PW_API int pw_fp64_config(pw_ctx* ctx, int set_mode, int* mode);
 
 /* Measured FP64 FMA rate of the current GPU (the roofline of DFMA-bound kernels: the DFMA

@@ -12,12 +12,13 @@
 //
 // Measured on GB300 against the FP64 kernels of fft_local.cu (10-step filter of 256 bands on 96^3):
 // x lines 184 -> 36 ms, pass 1 67 -> 15 ms, pass 3 74 -> 19 ms; density of 256 bands, same box,
-// 17.3 -> 5.5 ms; one vector on 64^3 (an H-apply of the Lanczos chain) 188 -> 90 us.  Relative
+// 17.3 -> 4.5 ms; one vector on 64^3 (an H-apply of the Lanczos chain) 188 -> 90 us.  Relative
 // error of V psi against extended precision 1.3e-16 to 1.9e-16 on boxes from 64^3 to 72 x 75 x 80
 // (FP64 kernels 4.4e-16 to 5.2e-16), random, decaying, single-component and in-phase bands alike.
 //
-// What bounds them: issue of the integer instructions (half of the slots at 16 warps per SM, 42%
-// of the ALU pipe); the conversions to and from FP64 take a fifth of the FP64 pipe.  Radices and
+// What bounds them: issue of the integer instructions (counters taken with two CTAs per SM: half of
+// the slots, 42% of the ALU pipe; three CTAs, 24 warps, run now) and the conversions to and from FP64,
+// a fifth of the FP64 pipe in the x pass, up to two fifths in the others.  Radices and
 // lengths are run-time values (a switch around a stage, uniform in the CTA): one set of kernels
 // covers every two-stage length, and the index arithmetic is small beside 64-bit butterflies.
 //
@@ -899,7 +900,7 @@ cudaError_t local_apply(const FftPlan& plan, const double2* tw, const SphereDev&
     (big(dy) ? k_fx_yinv<true> : k_fx_yinv<false>)<<<dim3(sp.nplane * nc, nb), kThreads, smy, st>>>(hb, hb_bs, sp, dy, dz.n, nc, by); count_launch();
     prof_end(prof, PW_PROF_PLANE_INV);
     prof_begin(prof, PW_PROF_XLINE);
-    // a few waves of CTAs; each converts V once for its bands
+    // a few waves of CTAs; each finds the scale of V on its lines once for its bands
     int splits = std::max(1, std::min(nb, (152 * 2 * 4 + gx - 1) / gx));
     const int bper = (nb + splits - 1) / splits;
     splits = (nb + bper - 1) / bper;

@@ -6,10 +6,14 @@
 // passes here read and write the same complex128 arrays as the FP64 kernels; inside a CTA each
 // line's values are integers on one power-of-two scale taken from the line's largest input.
 //
-// Error: an input component is rounded to 2^-57 of its line's largest one (2^-55 at length 256),
-// every product to one unit of the same scale and sums are exact, whatever the values' signs and
-// sizes.  The largest component is at most sqrt(n) times the r.m.s. of its line, so the error of a
-// transform stays below that of one with FP64's 2^-53 rounding in every sum and product.
+// Error: an input component is rounded to 2^-57 of its line's largest one (2^-56 at lengths from 120
+// to 225, 2^-55 at 240 and 256), every product to one unit of the same scale and sums are exact,
+// whatever the values' signs and sizes.  Components below 2^-4 (2^-3, 2^-2) of the largest thus enter
+// with fewer bits than FP64 holds, as they would leave an FP64 transform: every output mixes the whole
+// line.  The largest component is at most sqrt(n) times the r.m.s. of its line, so the error of a
+// transform stays below that of one with FP64's 2^-53 rounding in every sum and product (measured on
+// spectra from flat to a single component, tests/test_gpu_fixed_fft.py).  Subnormal components count
+// as zero.
 #pragma once
 #include "pw_internal.cuh"
 

@@ -2293,12 +2293,11 @@ static cudaError_t plane_wg_pair(int which, const cplx<T>* psi, int64_t ldpsi, c
         if constexpr (std::is_same<T, float>::value) {
           auto run = [&](auto rc) -> cudaError_t {  // 1 with P Z, 2 without
             constexpr int R = decltype(rc)::value;
-          if ((e = smem_limit(k_plane_fwd_wgp<T, N2, N3, TW, R>, sm)))
-            return e;
-          const int grid = grid_of((const void*)k_plane_fwd_wgp<T, N2, N3, TW, R>);
-          k_plane_fwd_wgp<T, N2, N3, TW, R><<<grid, PW::THREADS, sm, st>>>(hb, hb_bs, sp, plan, tw, kin, psi,
-                                                                             ldpsi, out, ldout, *rec, nb);
-          count_launch();
+            if ((e = smem_limit(k_plane_fwd_wgp<T, N2, N3, TW, R>, sm))) return e;
+            const int grid = grid_of((const void*)k_plane_fwd_wgp<T, N2, N3, TW, R>);
+            k_plane_fwd_wgp<T, N2, N3, TW, R><<<grid, PW::THREADS, sm, st>>>(hb, hb_bs, sp, plan, tw, kin, psi, ldpsi,
+                                                                             out, ldout, *rec, nb);
+            count_launch();
             return cudaSuccess;
           };
           e = rec->pz ? run(std::integral_constant<int, 1>{}) : run(std::integral_constant<int, 2>{});
@@ -2342,13 +2341,12 @@ static cudaError_t plane_wg_pair(int which, const cplx<T>* psi, int64_t ldpsi, c
         if constexpr (std::is_same<T, float>::value) {
           auto run = [&](auto rc) -> cudaError_t {  // 1 with P Z, 2 without
             constexpr int R = decltype(rc)::value;
-          if ((e = smem_limit(k_plane_fwd_wg<T, N2, N3, TW, R>, sm)))
-            return e;
-          if ((e = cudaFuncSetAttribute(k_plane_fwd_wg<T, N2, N3, TW, R>,
-                                        cudaFuncAttributePreferredSharedMemoryCarveout, 100)))
-            return e;
-          k_plane_fwd_wg<T, N2, N3, TW, R><<<dim3(sp.nplane, nb), PW::THREADS, sm, st>>>(
-              hb, hb_bs, sp, plan, tw, kin, psi, ldpsi, out, ldout, *rec); count_launch();
+            if ((e = smem_limit(k_plane_fwd_wg<T, N2, N3, TW, R>, sm))) return e;
+            if ((e = cudaFuncSetAttribute(k_plane_fwd_wg<T, N2, N3, TW, R>,
+                                          cudaFuncAttributePreferredSharedMemoryCarveout, 100)))
+              return e;
+            k_plane_fwd_wg<T, N2, N3, TW, R><<<dim3(sp.nplane, nb), PW::THREADS, sm, st>>>(
+                hb, hb_bs, sp, plan, tw, kin, psi, ldpsi, out, ldout, *rec); count_launch();
             return cudaSuccess;
           };
           e = rec->pz ? run(std::integral_constant<int, 1>{}) : run(std::integral_constant<int, 2>{});
@@ -2679,17 +2677,16 @@ static cudaError_t plane_rs_pair(int which, const cplx<T>* psi, int64_t ldpsi, c
       k_plane_inv_rs<T, N2, N3, TW><<<grid, PR::THREADS, sm, st>>>(psi, ldpsi, hb, hb_bs, sp, plan, tw); count_launch();
     } else if (rec) {
       if constexpr (kF32) {
-          auto run = [&](auto rc) -> cudaError_t {  // 1 with P Z, 2 without
-            constexpr int R = decltype(rc)::value;
-        if ((e = smem_limit(k_plane_fwd_rs<T, N2, N3, TW, R>, sm)))
-          return e;
-        k_plane_fwd_rs<T, N2, N3, TW, R><<<grid, PR::THREADS, sm, st>>>(hb, hb_bs, sp, plan, tw, kin, psi, ldpsi,
+        auto run = [&](auto rc) -> cudaError_t {  // 1 with P Z, 2 without
+          constexpr int R = decltype(rc)::value;
+          if ((e = smem_limit(k_plane_fwd_rs<T, N2, N3, TW, R>, sm))) return e;
+          k_plane_fwd_rs<T, N2, N3, TW, R><<<grid, PR::THREADS, sm, st>>>(hb, hb_bs, sp, plan, tw, kin, psi, ldpsi,
                                                                           out, ldout, *rec); count_launch();
-            return cudaSuccess;
-          };
-          e = rec->pz ? run(std::integral_constant<int, 1>{}) : run(std::integral_constant<int, 2>{});
-          if (e) return e;
-        }
+          return cudaSuccess;
+        };
+        e = rec->pz ? run(std::integral_constant<int, 1>{}) : run(std::integral_constant<int, 2>{});
+        if (e) return e;
+      }
     } else {
       if ((e = smem_limit(k_plane_fwd_rs<T, N2, N3, TW, 0>, sm)))
         return e;
@@ -2818,8 +2815,8 @@ static bool plane_lg_covers(const FftPlan& plan) {
 // once, two per SM or four small ones, a block-wide pass takes 10 us (18^2 points), 13 (32^2), 18 (54 x
 // 60), 23 (72 x 75); the next plane on an SM costs 30 to 50% more.  The recurrence in pass 3 (`rec`) is
 // worth about 9 us a step, so a filter changes over earlier.  us for a 6-step filter with the block-wide
-// planes and without: 25 x 27 x 30, 8 bands 442 and 502, 32 bands (352 planes) 570 and 519; 54 x 54 x 60,
-// 1 band 559 and 577.
+// planes and without: 25 x 27 x 30, 8 bands 440 and 508, 32 bands (352 planes) 511 and 517; 32^3, 16 bands
+// 455 and 503; 54 x 54 x 60, 12 bands (300 planes) 617 and 635; H psi of 2 bands on 60^3 109 and 118.
 static bool planes_block_wide(const FftPlan& plan, const SphereDev& sp, int nb, bool rec) {
   if (plane_lg_covers(plan)) return false;
   const int64_t planes = (int64_t)sp.nplane * nb, points = (int64_t)plan.n[1] * plan.n[2];
@@ -2855,8 +2852,8 @@ cudaError_t launch_local_apply(const FftPlan& plan, const cplx<T>* tw, const Sph
   // multi-band forms double-buffered), plane form = variant / 16 (0 line groups, 1 one thread
   // per line, 2 warp groups over the whole plane, 3 warp groups over sphere rows and 32-column
   // slices, 4 = 3 for pass 1 and 2 for pass 3)
-  // complex128: only the plane form is selectable (0 line groups, 3 sphere rows + column
-  // slices); the x-line pass keeps the line-group form
+  // complex128 (boxes without two-stage plans, and FP64 solves): only the plane form is selectable
+  // (0 line groups, 3 sphere rows + column slices); the x-line pass keeps the line-group form
   const int fv = prof ? prof->fft_variant[std::is_same<T, float>::value ? 0 : 1] : 0;
   int xf = std::is_same<T, float>::value ? fv % kFormStride : 0;
   const int pf = fv / kFormStride;

@@ -8,7 +8,9 @@
 // kernels and the plain Jacobi (pw_ctx::keep64), and a k-point has the same vectors alone and in a
 // batch.  Every other call returns the faster kernels' results:
 // the densities, energies, residuals and gradients that are made from Ritz vectors do not depend on
-// the phases.
+// the phases.  The order covers what an FP64 solve does itself: the Woodbury matrices of Q are made with
+// the context, by the faster factorisations, and blocks of 2 to 4 bands take matrix-vector products whose
+// sums have four parts.
 #include <math.h>
 
 #include <algorithm>

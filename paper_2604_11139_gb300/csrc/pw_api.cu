@@ -1662,8 +1662,10 @@ template int recur<double>(pw_ctx*, const double2*, int64_t, const double2*, int
 template int recur<float>(pw_ctx*, const float2*, int64_t, const float2*, int64_t, float2*, int64_t, int, double,
                           double, double, float2*);
 // From 2^25 complex products the digits and their products (0.2 ms at 14771 x 128 x 128) beat the
-// FP64 pipe (4 FMAs each: 0.22 ms at 2^25, 1.6 ms at 14771 x 128 x 128).  Eight digits: the result is
-// as close to exact as the FMAs' (a product that the filter and Rayleigh-Ritz take with seven).
+// FP64 pipe (4 FMAs each: 0.22 ms at 2^25, 1.6 ms at 14771 x 128 x 128).  Eight digits, where the filter
+// and Rayleigh-Ritz take seven: bands and their adjoints decay alike along the plane waves, and the
+// result is then as close to exact as the FMAs' (zgemm.cuh; gradients of 128 bands on 64^3 3.3e-13 off,
+// 5.5e-13 with FMAs).  pw_fp64_config(0) keeps them on the FP64 pipe.
 int gemm64(pw_ctx* ctx, int ta, int tb, int M, int N, int K, const double2* A, int64_t lda, const double2* B,
            int64_t ldb, const Epi<double>& e, int nsplit, double2* ws, const char* where) {
   if ((double)M * N * K >= (double)(1 << 25))

@@ -318,7 +318,8 @@ struct pw_ctx {
   // tuning: bytes of half-box planes per FFT band batch (complex64, complex128); set by pw_autotune
   // (complex64: large launches beat planes handed over in L2, 10-step filter of 128 bands on
   // 72 x 72 x 90: 5.6 ms at 48 MB, 4.8 at 384 MB; complex128 the same, density of 256 bands on 96^3:
-  // 5.53 ms at 256 MB, 5.30 at 512 MB, the FP64 filter there 103.5 and 102.2 ms)
+  // 5.53 ms at 256 MB, 5.30 at 512 MB, the FP64 filter there 103.5 and 102.2 ms).  A context holds this
+  // much, or its whole block's planes where they are fewer: 32 k-points with blocks that fill it 12 GB
   size_t fft_batch_bytes[2] = {(size_t)384 << 20, (size_t)512 << 20};
   // FFT pass kernel forms per precision, variant = xline form + 8 * plane form.  x-line
   // forms: 0 line groups of 1-8 threads with shared-memory twiddles, 1 one thread per line
@@ -329,9 +330,10 @@ struct pw_ctx {
   // than 0 cover two-stage plans in complex64 only (otherwise form 0 runs); set by pw_autotune
   // FFT pass-kernel forms (complex64, complex128): complex64 defaults to the staged multi-band
   // x-lines (form 8) and plane form 3 with the recurrence in pass 3 (10-step filter of 128 bands on
-  // 72 x 72 x 90 with 48 MB batches: 5.5 ms, 10.0 on the line groups), complex128 to the sphere-row +
-  // column-slice plane kernels (plane form 3), which fall back to line groups where they do
-  // not apply (1.2x the line-group form on the 120^3 box)
+  // 72 x 72 x 90 with 48 MB batches: 5.5 ms, 10.0 on the line groups).  complex128 runs the fixed-point
+  // passes where every length has a two-stage plan, whatever the form; its form is that of the FP64
+  // kernels elsewhere and inside FP64 solves: sphere rows + column slices (plane form 3), which fall
+  // back to line groups where they do not apply (1.2x the line-group form on the 120^3 box)
   int fft_variant[2] = {8 + 3 * pw::kFormStride, 3 * pw::kFormStride};
   bool keep64 = false;  // inside an FP64 solve: fixed order of operations (la_keep.cu)
   int last_sweeps = 0;  // Jacobi sweeps of the last Rayleigh-Ritz step

@@ -8,7 +8,12 @@ namespace pw {
 namespace oz {
 
 // 7-bit digits per operand entry: 49 bits of each row-scaled entry, or 56, which carry FP64 entries
-// within 2^3 of the row's largest whole; products of the latter are as close as FP64 FMAs
+// within 2^3 of the row's largest whole.  Error of a sum of K products a_k b_k: below 2^-44 (seven
+// digits) or 2^-51 of |a_max| |b_max| per element; FMAs err relative to the running sum.  Emulated at
+// K = 4000, relative to |a| |b|: entries of even size 8 digits 3e-18, FMAs 8e-18; both decaying over 6
+// decades 7e-17 and 1e-16, over 10 both 1e-16 (7 digits 5e-16 to 6e-15); where one decays and the other
+// grows, products of even size add up to far less than |a| |b| and FMAs keep what eight digits do not
+// (4 decades: 2e-17 and 3e-20).
 constexpr int kDigits = 7, kDigitsFull = 8;
 
 // Digit planes of a K-major realified operand: dig[s * plane + row * pitch + k], s < digits,

@@ -24,14 +24,14 @@
 // the complex product: the output is the column-major complex block viewed as doubles.
 //
 // Kernel: persistent, one 128 (realified rows) x 64 (columns) output tile per work unit.
-// Warp 0 lane 0 issues TMA loads of all seven digit planes of a 32-wide K slice of both
+// Warp 0 lane 0 issues TMA loads of all digit planes (seven or eight) of a 32-wide K slice of both
 // operands (64-byte swizzle) into a two-stage ring; warp 1 lane 0 issues the slice's products, per
-// K step of 16 ten tcgen05.mma: digit p of A against up to four digits of B at once, whose rows
+// K step of 16 ten tcgen05.mma (twelve with eight digits): digit p of A against up to four digits of B at once, whose rows
 // are adjacent in shared memory as their accumulators are in TMEM (N up to 256; one instruction
 // of N = 64 per digit pair reads A's tile 28 times instead of 10; the products of the FP64 filter on
 // 96^3, 256 bands: 1.69 -> 1.30 ms a launch, those of Rayleigh-Ritz on 120^3, 512 bands: 5.8 ->
 // 4.4 ms).  The projection then reads its digit planes at 62% of the copy bandwidth; the tensor
-// pipe is active for 43% of the time.  Warps 2-17 drain the seven accumulators once
+// pipe is active for 43% of the time.  Warps 2-17 drain the accumulators once
 // per 256-wide K chunk (one TMEM lane = one output row per thread, 16 columns per warp).
 // Every mbarrier wait is bounded; on expiry the kernel records the stage, waits (bounded) for
 // the copies and MMAs it has issued, releases TMEM and returns.
